@@ -158,16 +158,17 @@ opal_status opal_energy_momentum(const opal_sim* sim, int32_t sys, double* E, do
  * Those are callers whose device memory is all held by another allocator
  * (a caching allocator that has reserved the GPU's HBM), and callers that
  * must not synchronize the device while steps are in flight (cudaMalloc
- * and cudaFree may synchronize; this call only enqueues two kernels).
+ * and cudaFree may synchronize; this call only enqueues three kernels).
  *   n          bodies, 0 <= n <= 131072; a larger n returns OPAL_EINVAL and
- *              launches nothing (the scratch is a fixed 1024 x 13 doubles
- *              in device memory, one row per 128-body block).
+ *              launches nothing (the scratch is a fixed 4.3 MB of device
+ *              memory: partial sums, and each body's coordinates and mass
+ *              split into floats for the pair sum).
  *   G, M0      as in opal_params (finite, > 0).
  *   m[n], x[3n], v[3n]   masses, heliocentric positions and heliocentric
  *              velocities (row-major n x 3), device memory of the current
  *              device (or managed), 8-byte aligned; borrowed, not kept.
  *              Bodies with m = 0 contribute nothing.
- *   out[7]     device memory: E, L[3], P[3], written by the second kernel.
+ *   out[7]     device memory: E, L[3], P[3], written by the last kernel.
  *   stream     cudaStream_t the kernels go on (NULL: the legacy stream).
  * The call returns once the kernels are enqueued: synchronize the stream
  * before reading out.  Nothing has to be zeroed first: out and every

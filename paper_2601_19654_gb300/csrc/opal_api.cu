@@ -80,11 +80,9 @@ struct opal_sim {
     std::vector<int64_t> n_per_sys;
     std::vector<KickItem> items;
     std::vector<PairTile> tiles;
-    std::vector<int64_t> tile_off;
     KickItem* d_items = nullptr;
     PairTile* d_tiles = nullptr;
-    int64_t* d_tile_off = nullptr;
-    int kick_grid = 1, scan_grid = 1, confirm_grid = 1, bs_grid = 1, energy_grid = 1;
+    int kick_grid = 1, scan_grid = 1, confirm_grid = 1, bs_grid = 1;
     int kick_variant = 0;
     char kick_desc[256] = {0};
     int time_kick = 0;                       // graph records events around the kick
@@ -100,6 +98,7 @@ struct opal_sim {
     double* h_rec = nullptr;       // pinned host copies of the two (allocated at the first get_state)
     int* h_ralive = nullptr;
     double* d_en_body = nullptr;
+    float4 *d_en_a = nullptr, *d_en_b = nullptr;   // the energy's float pairs of every body
     double* d_en_pair = nullptr;
     double* d_en_out = nullptr;
     std::vector<void*> allocs;
@@ -240,7 +239,6 @@ void build_kick_items(opal_sim* s, int slots, int itile, bool jmajor) {
 
 void build_pair_tiles(opal_sim* s) {
     s->tiles.clear();
-    s->tile_off.assign(1, 0);
     for (size_t k = 0; k < s->sys.size(); k++) {
         const SysInfo& si = s->sys[k];
         // tile pairs (A, B >= A) with a big body in A: every pair with a big
@@ -254,7 +252,6 @@ void build_pair_tiles(opal_sim* s) {
                 t.j0 = si.off + b * kSeg;
                 s->tiles.push_back(t);
             }
-        s->tile_off.push_back((int64_t)s->tiles.size());
     }
 }
 
@@ -407,7 +404,6 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
     build_pair_tiles(s);
     const int64_t nt = std::max<int64_t>(1, (int64_t)s->tiles.size());
     s->scan_grid = (int)std::min<int64_t>(nt, (int64_t)s->nsm * 16);
-    s->energy_grid = (int)std::min<int64_t>(nt, (int64_t)s->nsm * 16);
     s->confirm_grid = s->nsm * 2;
     s->bs_grid = s->nsm * 4;
     const int64_t slots = max_slots;
@@ -522,7 +518,6 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
     TRYF(dalloc(s, &s->d_items, max_items));
     TRYF(dalloc(s, &s->d_tiles, s->tiles.size()));
     TRYF(dalloc(s, &d.tov, std::max<size_t>(1, s->tiles.size())));
-    TRYF(dalloc(s, &s->d_tile_off, s->tile_off.size()));
     {
         int64_t maxcap = 0;
         for (auto& si : s->sys) maxcap = std::max(maxcap, si.cap);
@@ -531,9 +526,11 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
         TRYF(dalloc(s, &s->d_exP, 3));
         TRYF(dalloc(s, &s->d_excnt, nsys));
     }
-    TRYF(dalloc(s, &s->d_en_body, 7 * (N / 128)));
-    TRYF(dalloc(s, &s->d_en_pair, s->tiles.size()));
-    TRYF(dalloc(s, &s->d_en_out, 8 * nsys));
+    TRYF(dalloc(s, &s->d_en_body, kEnSums * (N / 128)));
+    TRYF(dalloc(s, &s->d_en_a, N));
+    TRYF(dalloc(s, &s->d_en_b, N));
+    TRYF(dalloc(s, &s->d_en_pair, kEnMaxGrid));
+    TRYF(dalloc(s, &s->d_en_out, 8));
 
     // host staging in the padded SoA layout
     std::vector<double> hx(N), hy(N), hz(N), hvx(N, 0.0), hvy(N, 0.0), hvz(N, 0.0), hm(N, 0.0), hR(N, 0.0);
@@ -565,7 +562,6 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
     CKF(up(d.alive, halive.data(), N * 4)); CKF(up(d.body_sys, hsys.data(), N * 4));
     CKF(up(d.label, hlabel.data(), N * 4));
     CKF(up(s->d_tiles, s->tiles.data(), s->tiles.size() * sizeof(PairTile)));
-    CKF(up(s->d_tile_off, s->tile_off.data(), s->tile_off.size() * sizeof(int64_t)));
     CKF(cudaMemsetAsync(d.ctl, 0, sizeof(Ctl), s->stream));
     CKF(cudaMemsetAsync(d.E_lost, 0, nsys * 8, s->stream));
     CKF(cudaMemsetAsync(d.ax, 0, N * 8, s->stream));
@@ -959,11 +955,11 @@ opal_status opal_energy_momentum(const opal_sim* cs, int32_t sys, double* E, dou
     opal_sim* s = const_cast<opal_sim*>(cs);
     if (!s) return set_err(g_err, "sim is NULL"), OPAL_EINVAL;
     if (sys < 0 || sys >= s->d.nsys) return set_err(s->err, "no system %d", sys), OPAL_EINVAL;
-    launch_energy(s->d, s->d_tiles, (int64_t)s->tiles.size(), s->d_tile_off, s->d_en_pair, s->d_en_body,
-                  s->d_en_out, s->energy_grid, s->stream);
+    launch_energy(s->d, sys, s->sys[sys], s->nsm, s->d_en_a, s->d_en_b, s->d_en_pair, s->d_en_body, s->d_en_out,
+                  s->stream);
     CK(cudaGetLastError());
     double o[8];
-    CK(cudaMemcpyAsync(o, s->d_en_out + 8 * sys, sizeof(o), cudaMemcpyDeviceToHost, s->stream));
+    CK(cudaMemcpyAsync(o, s->d_en_out, sizeof(o), cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
     if (E) *E = o[0];
     if (L) { L[0] = o[1]; L[1] = o[2]; L[2] = o[3]; }

@@ -253,15 +253,18 @@ __global__ void __launch_bounds__(32 * kRowWarps, 4) k_kick_rows(Dev d) {
     const int b = MIXED ? d.csorted[p] : (int)p;
     const SysInfo si = d.sys[d.body_sys[p0]];
     const int64_t local = p - si.off;
+    // rows of this body (FP64 form, by body index: big and small bodies have their own number, padding none)
+    const int nrow = MIXED || local < si.nb ? si.nchunk : (local < si.n ? si.nchunk_small : 0);
+    const int nmax = MIXED ? si.nchunk : max(si.nchunk, si.nchunk_small);
     T ax = A::zero(), ay = A::zero(), az = A::zero();
 #pragma unroll 1
-    for (int c0 = kRowsPerWarp * gw; c0 < si.nchunk; c0 += kRowsPerWarp * G) {
+    for (int c0 = kRowsPerWarp * gw; c0 < nmax; c0 += kRowsPerWarp * G) {
         T bx[kRowsPerWarp], by[kRowsPerWarp], bz[kRowsPerWarp];
 #pragma unroll
         for (int u = 0; u < kRowsPerWarp; u++) {
             const int c = c0 + u;
             const int64_t slot = si.slot0 + (int64_t)c * si.cap + local;
-            const bool in = c < si.nchunk;
+            const bool in = c < nrow;
             bx[u] = in ? A::load(d.pacc_x, slot) : A::zero();
             by[u] = in ? A::load(d.pacc_y, slot) : A::zero();
             bz[u] = in ? A::load(d.pacc_z, slot) : A::zero();

@@ -432,14 +432,102 @@ __global__ void __launch_bounds__(T, MINB) k_kick_mixed(Dev d, const KickItem* _
     queue_done(d);
 }
 
-template <int T>
-__global__ void __launch_bounds__(T) k_kick_fp64(Dev d, const KickItem* __restrict__ items, int64_t nitems) {
+// FP64 form.  The FP64 pipe bounds it (a warp's FP64 instruction holds an
+// SM's pipe for 16 cycles, 1/62 of the FP32 rate), so what counts is FP64
+// instructions a pair; shuffles and integer tests are free beside it.
+//  - Two big bodies: a pair's separation and 1/r^3 serve both of them (12
+//    instructions, then 4 for each side: 20 a pair of bodies where the
+//    one-sided sum took 2 x 20).  A warp holds 32 i-bodies, one a lane, and 32
+//    j-bodies that rotate through the lanes with their sums; after 32 steps
+//    every pair has met and the j-sums are back in their lanes.
+//  - 1/r^3 from the approximate FP64 reciprocal square root y of the hardware
+//    (20 bits): y^2 is exact, d = 1 - r^2 y^2 measured below 1.9e-6 over the
+//    exponents, and 1/r^3 = y^3 (1 - d)^(-3/2) = y^3 (1 + d (3/2 + 15/8 d))
+//    with a next term below 2^-55 (6 instructions; the rounded reciprocal
+//    square root of the library and its cube took about 10).
+//  - Near pairs (the changeover, coincidence, the body itself) are those
+//    closer than the larger critical radius of the two, tested on the high
+//    words of the squares; the test was against twice the system's largest
+//    radius, which a giant planet spreads over most of a system.
+// Kick alone: 16384-body disk 8.74 to 4.94 ms (4.2e6 warp steps x 20 FP64
+// instructions x 16 cycles on 152 SMs are 4.3 ms at 2.07 GHz); 1001 bodies
+// 391 to 33 us (528 one-warp items where 32 blocks held 32 SMs); 301
+// big and 40000 small bodies 1753 to 427 us.  Errors against extended
+// precision: 3e-16 rms of a body's acceleration (5e-16 before).
+// Work items: a pair of super-tiles (A, B >= A) of the big bodies; row B of the
+// partial buffer gets A's sums, row A gets B's.  A super-tile is g tiles of W x
+// 32 bodies (W warps a block; g = 1 up to 128 super-tiles, more bodies take
+// larger g, which bounds the buffer at 128 rows or so).  The warps of a
+// block take the j-tile's 32-body parts in turn, a barrier between turns, so
+// that j-sums are added in shared memory in a fixed order.  Small bodies
+// are sources of nothing: their items are one-sided, an i-tile against a
+// run of the big bodies.
+constexpr double kKickParked = 1.0e150;   // coordinate of lanes without a body (finite squares)
+
+struct KickJ {
+    double x, y, z, m;
+    int rc2h;   // high word of rc^2 (at least that of 1e-300, so that r = 0 counts as near)
+};
+
+__device__ __forceinline__ KickJ kick_load(const Dev& d, int64_t b, bool in) {
+    KickJ r{kKickParked, kKickParked, kKickParked, 0.0, 0};
+    if (in) {
+        const double rc = d.rc[b];
+        r = KickJ{d.x[b], d.y[b], d.z[b], d.m[b], __double2hiint(fmax(rc * rc, 1e-300))};
+    }
+    return r;
+}
+
+// the 32 steps of a warp's i-bodies (a, one a lane) against 32 j-bodies (j, from
+// jb on): sums of m_j K (x_j - x_i) / r^3 into ai, and with SYM the opposite
+// ones into aj (a lane's own j)
+template <bool SYM>
+__device__ __forceinline__ void kick_turn(const Dev& d, const KickJ& a, double rci, KickJ j, int64_t jb, int form,
+                                          double (&ai)[3], double (&aj)[3]) {
+    const int lane = threadIdx.x & 31, next = (lane + 1) & 31;
+#pragma unroll 2
+    for (int k = 0; k < 32; k++) {
+        const double dx = j.x - a.x, dy = j.y - a.y, dz = j.z - a.z;
+        const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+        double s;
+        if ((unsigned)__double2hiint(r2) <= (unsigned)max(a.rc2h, j.rc2h)) {   // (a NaN is not near)
+            const int64_t b = jb + ((lane + k) & 31);
+            s = slow_pair_d(r2, 1.0, rci, j.rc2h ? d.rc[b] : 0.0, form);
+        } else {
+            double y;
+            asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));
+            const double y2 = y * y, e = fma(-r2, y2, 1.0);
+            const double y3 = y2 * y;
+            s = fma(y3 * e, fma(e, 1.875, 1.5), y3);
+        }
+        const double ti = j.m * s;
+        ai[0] = fma(ti, dx, ai[0]);
+        ai[1] = fma(ti, dy, ai[1]);
+        ai[2] = fma(ti, dz, ai[2]);
+        if (SYM) {
+            const double tj = -(a.m * s);
+            aj[0] = __shfl_sync(0xffffffffu, fma(tj, dx, aj[0]), next);
+            aj[1] = __shfl_sync(0xffffffffu, fma(tj, dy, aj[1]), next);
+            aj[2] = __shfl_sync(0xffffffffu, fma(tj, dz, aj[2]), next);
+        }
+        j.x = __shfl_sync(0xffffffffu, j.x, next);
+        j.y = __shfl_sync(0xffffffffu, j.y, next);
+        j.z = __shfl_sync(0xffffffffu, j.z, next);
+        j.m = __shfl_sync(0xffffffffu, j.m, next);
+        j.rc2h = __shfl_sync(0xffffffffu, j.rc2h, next);
+    }
+}
+
+template <int W>
+__global__ void __launch_bounds__(32 * W) k_kick_fp64(Dev d, const KickItem* __restrict__ items, int64_t nitems) {
     OPAL_TIMELINE_SCOPE(kTlKick);
     if (d.gated && !d.ctl->reprime) return;   // the re-evaluation after a removal, with none
-    __shared__ D4 sj[kJTile];
+    constexpr int S = 32 * W;
+    extern __shared__ double kick_sj[];       // [3][bodies of a super-tile]: the j side's sums
     __shared__ int s_item;
     if (d.ctl->status) return;
     const int form = d.p.changeover;
+    const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
     for (;;) {
         __syncthreads();
         if (threadIdx.x == 0) s_item = atomicAdd(&d.ctl->kick_next, 1);
@@ -448,42 +536,74 @@ __global__ void __launch_bounds__(T) k_kick_fp64(Dev d, const KickItem* __restri
         if (it >= nitems) break;
         const KickItem w = items[it];
         const SysInfo si = d.sys[w.sys];
-        const double rcm = (double)d.rcmax[w.sys];
-        for (int64_t ib = w.i0; ib < w.i1; ib += w.istep) {
-        const int64_t i = ib + threadIdx.x;
-        const double xi = d.x[i], yi = d.y[i], zi = d.z[i], rci = d.rc[i];
-        double t = 2.0 * (rci + rcm);
-        const double thr = fmax(t * t, 1e-300);
-        double ax = 0.0, ay = 0.0, az = 0.0;
-        for (int64_t jb = w.j0; jb < w.j1; jb += kJTile) {
-            const int nj = (int)min((int64_t)kJTile, w.j1 - jb);
-            __syncthreads();
-            for (int k = threadIdx.x; k < nj; k += T) {
-                int64_t j = jb + k;
-                sj[k] = D4{d.x[j], d.y[j], d.z[j], d.m[j]};
+        if (w.istep == 0) {   // small bodies: one-sided, an i-tile against a run of the big ones
+            const int64_t i = w.i0 + threadIdx.x;
+            const bool in = i < w.i1;
+            double ai[3] = {0.0, 0.0, 0.0}, none[3] = {0.0, 0.0, 0.0};
+            if (w.i0 + 32 * wq < w.i1) {
+                const KickJ a = kick_load(d, i, in);
+                const double rci = in ? d.rc[i] : 0.0;
+                for (int64_t jb = w.j0; jb < w.j1; jb += 32)
+                    kick_turn<false>(d, a, rci, kick_load(d, jb + lane, jb + lane < w.j1), jb, form, ai, none);
             }
-            __syncthreads();
-#pragma unroll 2
-            for (int jj = 0; jj < nj; jj++) {
-                const D4 pj = sj[jj];
-                double dx = pj.x - xi, dy = pj.y - yi, dz = pj.z - zi;
-                double r2 = dx * dx + dy * dy + dz * dz;
-                double s;
-                if (r2 < thr) {
-                    s = slow_pair_d(r2, pj.w, rci, d.rc[jb + jj], form);
-                } else {
-                    double ri = rsqrt(r2);
-                    s = (pj.w * ri) * (ri * ri);
+            if (in) {
+                const int64_t slot = si.slot0 + (int64_t)w.chunk * si.cap + (i - si.off);
+                d.pacc_x[slot] = ai[0];
+                d.pacc_y[slot] = ai[1];
+                d.pacc_z[slot] = ai[2];
+            }
+            continue;
+        }
+        // super-tiles A = [i0, i1) and B = [j0, j1) of w.istep bodies each
+        const bool own = w.i0 == w.j0;
+        const int nj = (int)(w.j1 - w.j0);
+        for (int k = threadIdx.x; k < nj; k += S)
+            for (int c = 0; c < 3; c++) kick_sj[c * w.istep + k] = 0.0;
+        __syncthreads();
+        for (int64_t ib = w.i0; ib < w.i1; ib += S) {
+            const int64_t i = ib + threadIdx.x;
+            const bool in = i < w.i1, some = ib + 32 * wq < w.i1;
+            const KickJ a = kick_load(d, i, in);
+            const double rci = in ? d.rc[i] : 0.0;
+            double ai[3] = {0.0, 0.0, 0.0};
+            for (int64_t jt = own ? ib : w.j0; jt < w.j1; jt += S) {
+                const bool one = own && jt == ib;   // a tile against itself: one-sided
+                for (int p = 0; p < W; p++) {
+                    const int64_t jb = jt + 32 * ((wq + p) % W);
+                    if (some && jb < w.j1) {
+                        const KickJ j = kick_load(d, jb + lane, jb + lane < w.j1);
+                        double aj[3] = {0.0, 0.0, 0.0};
+                        if (one) {
+                            kick_turn<false>(d, a, rci, j, jb, form, ai, aj);
+                        } else {
+                            kick_turn<true>(d, a, rci, j, jb, form, ai, aj);
+                            const int q = (int)(jb - w.j0) + lane;
+                            if (q < nj)
+                                for (int c = 0; c < 3; c++) kick_sj[c * w.istep + q] += aj[c];
+                        }
+                    }
+                    if (W > 1) __syncthreads();   // the next turn's warp adds to these sums
+                    else __syncwarp();
                 }
-                ax += s * dx;
-                ay += s * dy;
-                az += s * dz;
+            }
+            if (!in) continue;   // (no barrier below within this loop's turn)
+            if (own) {
+                const int q = (int)(i - w.j0);
+                for (int c = 0; c < 3; c++) kick_sj[c * w.istep + q] += ai[c];
+            } else {
+                const int64_t slot = si.slot0 + (int64_t)w.chunk * si.cap + (i - si.off);
+                d.pacc_x[slot] = ai[0];
+                d.pacc_y[slot] = ai[1];
+                d.pacc_z[slot] = ai[2];
             }
         }
-        int64_t slot = si.slot0 + (int64_t)w.chunk * si.cap + (i - si.off);
-        d.pacc_x[slot] = ax;
-        d.pacc_y[slot] = ay;
-        d.pacc_z[slot] = az;
+        __syncthreads();
+        const int64_t row = (w.i0 - si.off) / w.istep;
+        for (int k = threadIdx.x; k < nj; k += S) {
+            const int64_t slot = si.slot0 + row * si.cap + (w.j0 + k - si.off);
+            d.pacc_x[slot] = kick_sj[k];
+            d.pacc_y[slot] = kick_sj[w.istep + k];
+            d.pacc_z[slot] = kick_sj[2 * w.istep + k];
         }
     }
     queue_done(d);
@@ -850,7 +970,6 @@ struct KickVariant {
     const char* name;
     int threads;
     int ni;           // i-bodies per thread: an item's i-tile is threads x ni bodies
-    bool jmajor;      // items: a j-tile against a run of i-tiles (else an i-tile against a j-chunk)
     void (*launch)(const Dev&, const KickItem*, int64_t, int, cudaStream_t);
     int (*occupancy)();
 };
@@ -865,33 +984,35 @@ int occ_mixed() {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_kick_mixed<T, NI, MINB>, T, 0);
     return nb;
 }
-template <int T>
+template <int W>
 void launch_fp64(const Dev& d, const KickItem* items, int64_t nitems, int grid, cudaStream_t s) {
-    k_kick_fp64<T><<<grid, T, 0, s>>>(d, items, nitems);
+    k_kick_fp64<W><<<grid, 32 * W, d.kick_smem, s>>>(d, items, nitems);
 }
-template <int T>
+// Blocks an SM of the FP64 form: 4 of four warps 4.94 ms on the 16384-body
+// disk, 3: 5.12, 2: 4.99, 5: 4.97 (the pipe is full with two warps a scheduler).
+template <int W>
 int occ_fp64() {
-    int nb = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_kick_fp64<T>, T, 0);
-    return nb;
+    cudaFuncSetAttribute(k_kick_fp64<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, kKickSuperMax * W * 32 * 24);
+    return 16 / W;
 }
 
 static const KickVariant kMixed[] = {
-    {"mixed t128 i1", 128, 1, true, launch_mixed<128, 1, 7>, occ_mixed<128, 1, 7>},
-    {"mixed t128 i1 6", 128, 1, true, launch_mixed<128, 1, 6>, occ_mixed<128, 1, 6>},
-    {"mixed t128 i1 8", 128, 1, true, launch_mixed<128, 1, 8>, occ_mixed<128, 1, 8>},
-    {"mixed t64 i2", 64, 2, true, launch_mixed<64, 2, 8>, occ_mixed<64, 2, 8>},
-    {"mixed t128 i2", 128, 2, true, launch_mixed<128, 2, 5>, occ_mixed<128, 2, 5>},
+    {"mixed t128 i1", 128, 1, launch_mixed<128, 1, 7>, occ_mixed<128, 1, 7>},
+    {"mixed t128 i1 6", 128, 1, launch_mixed<128, 1, 6>, occ_mixed<128, 1, 6>},
+    {"mixed t128 i1 8", 128, 1, launch_mixed<128, 1, 8>, occ_mixed<128, 1, 8>},
+    {"mixed t64 i2", 64, 2, launch_mixed<64, 2, 8>, occ_mixed<64, 2, 8>},
+    {"mixed t128 i2", 128, 2, launch_mixed<128, 2, 5>, occ_mixed<128, 2, 5>},
 };
 static const KickVariant kFp64[] = {
-    {"fp64 t128", 128, 1, false, launch_fp64<128>, occ_fp64<128>},
+    {"fp64 w1", 32, 1, launch_fp64<1>, occ_fp64<1>},
+    {"fp64 w2", 64, 1, launch_fp64<2>, occ_fp64<2>},
+    {"fp64 w4", 128, 1, launch_fp64<4>, occ_fp64<4>},
 };
 
 int kick_num_variants(int precision) {
     return precision == 1 ? (int)(sizeof(kMixed) / sizeof(kMixed[0])) : (int)(sizeof(kFp64) / sizeof(kFp64[0]));
 }
 const char* kick_variant_name(int precision, int v) { return precision == 1 ? kMixed[v].name : kFp64[v].name; }
-bool kick_jmajor(int precision, int v) { return precision == 1 ? kMixed[v].jmajor : kFp64[v].jmajor; }
 int kick_itile(int precision, int v) {
     const KickVariant& k = precision == 1 ? kMixed[v] : kFp64[v];
     return k.threads * k.ni;

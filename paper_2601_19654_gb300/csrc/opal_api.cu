@@ -143,22 +143,16 @@ bool finite_all(const double* a, int64_t n) {
     return true;
 }
 
-// The kick's work list.  Only a system's first nb places (its big bodies)
+// The mixed kick's work list.  Only a system's first nb places (its big bodies)
 // are sources: j runs over them (small bodies follow them, in storage and in
 // the sorted order alike); i runs over all cap places.  Items are taken from
 // a queue, largest first.
-//  - i-major (jmajor false): an i-tile of itile bodies against a j-chunk,
-//    chunk edges on whole j-tiles, about eight items per resident block;
-//    the chunk's partial row.
-//  - j-major: one j-tile (staged once) against a run of i-tiles; the j-tile
-//    index is the partial row.  The (i-tile, j-tile) units are grouped into
-//    runs of 4 while more than four grids' worth of units remain (slots =
-//    the blocks of the launch), then of 2 while more than two remain, then
-//    single units, so that the queue ends on the smallest items.
-void build_kick_items(opal_sim* s, int slots, int itile, bool jmajor) {
-    double work = 0;
-    for (auto& si : s->sys) work += (double)si.cap * (double)si.nb;
-    const double target = std::max(1.0, work / (8.0 * std::max(1, slots)));
+// An item is one j-tile (staged once) against a run of i-tiles; the j-tile
+// index is the partial row.  The (i-tile, j-tile) units are grouped into
+// runs of 4 while more than four grids' worth of units remain (slots = the
+// blocks of the launch), then of 2 while more than two remain, then single
+// units, so that the queue ends on the smallest items.
+void build_kick_items_mixed(opal_sim* s, int slots, int itile) {
     s->items.clear();
     int64_t slot = 0, units = 0;
     for (auto& si : s->sys) units += (si.cap / itile) * ((si.nb + kKickJTile - 1) / kKickJTile);
@@ -167,67 +161,44 @@ void build_kick_items(opal_sim* s, int slots, int itile, bool jmajor) {
         SysInfo& si = s->sys[k];
         const int64_t itiles = si.cap / itile;
         const int64_t jtiles = (si.nb + kKickJTile - 1) / kKickJTile;
-        if (jmajor) {
-            si.nchunk = (int32_t)std::max<int64_t>(1, jtiles);
-            si.slot0 = slot;
-            slot += (int64_t)si.nchunk * si.cap;
-            for (int64_t t = 0; t < jtiles; t++) {
-                const int64_t j0 = si.off + t * kKickJTile, j1 = si.off + std::min(si.nb, (t + 1) * kKickJTile);
-                for (int64_t a = 0; a < itiles;) {
-                    int64_t run = left > 4 * (int64_t)slots ? 4 : (left > 2 * (int64_t)slots ? 2 : 1);
-                    run = std::min(run, itiles - a);
-                    // the run's i-tiles a + u * S (u < run) for a block of run * S tiles,
-                    // S = the block's stride: spatial neighbours go to different items
-                    const int64_t span = std::min(itiles - a, (itiles - a) / run * run);
-                    const int64_t S = std::max<int64_t>(1, span / run);
-                    for (int64_t b = 0; b < S; b++) {
-                        KickItem it{};
-                        it.sys = (int32_t)k;
-                        it.chunk = (int32_t)t;
-                        it.i0 = si.off + (a + b) * itile;
-                        it.istep = S * itile;
-                        it.i1 = it.i0 + run * S * itile;
-                        it.j0 = j0;
-                        it.j1 = j1;
-                        s->items.push_back(it);
-                        left -= run;
-                    }
-                    a += run * S;
-                }
-            }
-            if (jtiles == 0) {
-                // no sources: one empty item per i-tile still writes the zero partial row
-                for (int64_t a = 0; a < itiles; a++) {
+        si.nchunk = (int32_t)std::max<int64_t>(1, jtiles);
+        si.nchunk_small = si.nchunk;
+        si.slot0 = slot;
+        slot += (int64_t)si.nchunk * si.cap;
+        for (int64_t t = 0; t < jtiles; t++) {
+            const int64_t j0 = si.off + t * kKickJTile, j1 = si.off + std::min(si.nb, (t + 1) * kKickJTile);
+            for (int64_t a = 0; a < itiles;) {
+                int64_t run = left > 4 * (int64_t)slots ? 4 : (left > 2 * (int64_t)slots ? 2 : 1);
+                run = std::min(run, itiles - a);
+                // the run's i-tiles a + u * S (u < run) for a block of run * S tiles,
+                // S = the block's stride: spatial neighbours go to different items
+                const int64_t span = std::min(itiles - a, (itiles - a) / run * run);
+                const int64_t S = std::max<int64_t>(1, span / run);
+                for (int64_t b = 0; b < S; b++) {
                     KickItem it{};
                     it.sys = (int32_t)k;
-                    it.chunk = 0;
-                    it.i0 = si.off + a * itile;
-                    it.i1 = it.i0 + itile;
-                    it.istep = itile;
-                    it.j0 = it.j1 = si.off;
+                    it.chunk = (int32_t)t;
+                    it.i0 = si.off + (a + b) * itile;
+                    it.istep = S * itile;
+                    it.i1 = it.i0 + run * S * itile;
+                    it.j0 = j0;
+                    it.j1 = j1;
                     s->items.push_back(it);
+                    left -= run;
                 }
+                a += run * S;
             }
-            continue;
         }
-        const double w_tile = (double)itile * (double)si.nb;
-        int64_t nchunk = (int64_t)std::llround(w_tile / target);
-        nchunk = std::max<int64_t>(1, std::min<int64_t>(nchunk, jtiles));
-        si.nchunk = (int32_t)nchunk;
-        si.slot0 = slot;
-        slot += nchunk * si.cap;
-        for (int64_t c = 0; c < nchunk; c++) {
-            const int64_t t0 = jtiles * c / nchunk, t1 = jtiles * (c + 1) / nchunk;
-            const int64_t j0 = si.off + t0 * kKickJTile, j1 = si.off + std::min(si.nb, t1 * kKickJTile);
-            for (int64_t t = 0; t < itiles; t++) {
+        if (jtiles == 0) {
+            // no sources: one empty item per i-tile still writes the zero partial row
+            for (int64_t a = 0; a < itiles; a++) {
                 KickItem it{};
                 it.sys = (int32_t)k;
-                it.chunk = (int32_t)c;
-                it.i0 = si.off + t * itile;
+                it.chunk = 0;
+                it.i0 = si.off + a * itile;
                 it.i1 = it.i0 + itile;
                 it.istep = itile;
-                it.j0 = j0;
-                it.j1 = j1;
+                it.j0 = it.j1 = si.off;
                 s->items.push_back(it);
             }
         }
@@ -235,6 +206,79 @@ void build_kick_items(opal_sim* s, int slots, int itile, bool jmajor) {
     std::stable_sort(s->items.begin(), s->items.end(), [](const KickItem& a, const KickItem& b) {
         return (a.i1 - a.i0) * (a.j1 - a.j0) > (b.i1 - b.i0) * (b.j1 - b.j0);
     });
+}
+
+// The FP64 kick's work list (see k_kick_fp64) for blocks of W warps: pairs of
+// super-tiles of each system's big bodies, and i-tiles of its small bodies
+// against runs of the big ones (the whole of them once that gives every SM
+// eight items: 301 big and 40000 small bodies 427 us, in two runs 456).  d.kick_smem gets the launch's shared memory.
+void build_kick_items_fp64(opal_sim* s, int W) {
+    s->items.clear();
+    const int64_t S = 32 * W;
+    int64_t slot = 0, small_tiles = 0, widest = 0;
+    for (auto& si : s->sys) small_tiles += (si.n - si.nb + S - 1) / S;
+    for (size_t k = 0; k < s->sys.size(); k++) {
+        SysInfo& si = s->sys[k];
+        const int64_t g = std::min<int64_t>(kKickSuperMax, std::max<int64_t>(1, (si.nb + 128 * S - 1) / (128 * S)));
+        const int64_t step = g * S, T = (si.nb + step - 1) / step;
+        if (T > 0) widest = std::max(widest, step);
+        int64_t runs = 0;
+        if (si.nb > 0 && si.n > si.nb)
+            runs = std::max<int64_t>(1, std::min<int64_t>((si.nb + 127) / 128, 8 * s->nsm / std::max<int64_t>(1, small_tiles)));
+        si.nchunk = (int32_t)T;
+        si.nchunk_small = (int32_t)runs;
+        si.slot0 = slot;
+        slot += std::max<int64_t>(T, runs) * si.cap;
+        for (int64_t a = 0; a < T; a++)
+            for (int64_t b = a; b < T; b++) {
+                KickItem it{};
+                it.sys = (int32_t)k;
+                it.chunk = (int32_t)b;
+                it.i0 = si.off + a * step;
+                it.i1 = si.off + std::min(si.nb, (a + 1) * step);
+                it.j0 = si.off + b * step;
+                it.j1 = si.off + std::min(si.nb, (b + 1) * step);
+                it.istep = step;
+                s->items.push_back(it);
+            }
+        for (int64_t r = 0; r < runs; r++)
+            for (int64_t a = si.nb; a < si.n; a += S) {
+                KickItem it{};
+                it.sys = (int32_t)k;
+                it.chunk = (int32_t)r;
+                it.i0 = si.off + a;
+                it.i1 = si.off + std::min(si.n, a + S);
+                it.j0 = si.off + si.nb * r / runs;
+                it.j1 = si.off + si.nb * (r + 1) / runs;
+                it.istep = 0;
+                s->items.push_back(it);
+            }
+    }
+    std::stable_sort(s->items.begin(), s->items.end(), [](const KickItem& a, const KickItem& b) {
+        return (a.i1 - a.i0) * (a.j1 - a.j0) > (b.i1 - b.i0) * (b.j1 - b.j0);
+    });
+    s->d.kick_smem = (int)(widest * 24);
+}
+
+void build_kick_items(opal_sim* s, int precision, int variant, int slots) {
+    if (precision == 1) build_kick_items_mixed(s, slots, kick_itile(precision, variant));
+    else build_kick_items_fp64(s, kick_threads(precision, variant) / 32);
+}
+
+// Warps a block of the FP64 kick: as many (4, 2 or 1: tiles of 128, 64 or 32
+// bodies) as leave every SM 16 items, whose last round then idles little
+// (1001 bodies: 33, 53 and 103 us with 1, 2 and 4; 16384: 5.09, 4.99 and 4.94 ms).
+int fp64_variant(const opal_sim* s) {
+    for (int v = kick_num_variants(0) - 1; v > 0; v--) {
+        const int64_t S = kick_threads(0, v);
+        int64_t items = 0;
+        for (auto& si : s->sys) {
+            const int64_t T = (si.nb + S - 1) / S;
+            items += T * (T + 1) / 2 + (si.nb > 0 ? (si.n - si.nb + S - 1) / S : 0);
+        }
+        if (items >= 16 * (int64_t)s->nsm) return v;
+    }
+    return 0;
 }
 
 void build_pair_tiles(opal_sim* s) {
@@ -385,20 +429,26 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
     d.huge_wait_ns = kHugeWaitNs;
     d.huge_hold = 0;
     d.nseg_tot = N / kSeg;
-    // kick variants: the work list of each, and the largest partial buffer any needs
+    // kick variants: the work list of each, and the largest partial buffer any
+    // needs.  The FP64 form's is chosen by the sizes, the mixed form's by timing.
     const int nvar = kick_num_variants(p->precision);
+    const char* force = getenv("OPAL_KICK_VARIANT");
+    int only = -1;
+    if (force) only = std::max(0, std::min(nvar - 1, atoi(force)));
+    else if (p->precision == 0) only = fp64_variant(s);
     std::vector<std::vector<KickItem>> var_items(nvar);
     std::vector<std::vector<SysInfo>> var_sys(nvar);
     std::vector<int> var_grid(nvar);
     int64_t max_slots = 0;
     for (int v = 0; v < nvar; v++) {
+        if (only >= 0 && v != only) continue;
         int occ = std::max(1, kick_occupancy(p->precision, v));
-        build_kick_items(s, s->nsm * occ, kick_itile(p->precision, v), kick_jmajor(p->precision, v));
+        build_kick_items(s, p->precision, v, s->nsm * occ);
         var_items[v] = s->items;
         var_sys[v] = s->sys;
         var_grid[v] = (int)std::min<int64_t>((int64_t)s->items.size(), (int64_t)s->nsm * occ);
         int64_t sl = 0;
-        for (auto& si : s->sys) sl += (int64_t)si.nchunk * si.cap;
+        for (auto& si : s->sys) sl += (int64_t)std::max(si.nchunk, si.nchunk_small) * si.cap;
         max_slots = std::max(max_slots, sl);
     }
     build_pair_tiles(s);
@@ -570,7 +620,7 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
     CKF(cudaMemsetAsync(d.rcmax, 0, nsys * 4, s->stream));
     // democratic heliocentric velocities, critical radii (offsets and
     // capacities are the same in every variant's system table)
-    CKF(up(d.sys, var_sys[0].data(), nsys * sizeof(SysInfo)));
+    CKF(up(d.sys, var_sys[only >= 0 ? only : 0].data(), nsys * sizeof(SysInfo)));
     launch_to_dh(d, s->stream);
     launch_prime(d, s->stream);
     // a spatially sorted body order for the kick (each step's scan sorts again)
@@ -586,13 +636,12 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
         // graph, with every block it fits 144 us, the encounter kernel the same)
         auto graph_blocks = [&](int v) { return std::max(1, kick_occupancy(p->precision, v)); };
         int best = 0;
-        const char* force = getenv("OPAL_KICK_VARIANT");
         double work = 0;
         for (auto& si : s->sys) work += (double)si.cap * (double)si.n;
         double best_ms = -1;
         std::vector<double> var_ms(nvar, -1.0);
-        if (force) {
-            best = std::max(0, std::min(nvar - 1, atoi(force)));
+        if (only >= 0) {
+            best = only;
         } else if (nvar > 1 && work >= 4.0e6) {
             launch_kick_stage(d, P.precision, s->stream);
             cudaEvent_t e0, e1;
@@ -633,10 +682,11 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
             }
         }
         s->kick_variant = best;
-        s->kick_grid = (int)std::min<int64_t>((int64_t)var_items[best].size(), (int64_t)s->nsm * graph_blocks(best));
+        s->kick_grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)var_items[best].size(), (int64_t)s->nsm * graph_blocks(best)));
         // the chosen shape's work list, its item sizes scheduled for the blocks it runs with
-        build_kick_items(s, s->kick_grid, kick_itile(p->precision, best), kick_jmajor(p->precision, best));
-        s->kick_grid = (int)std::min<int64_t>((int64_t)s->items.size(), (int64_t)s->nsm * graph_blocks(best));
+        build_kick_items(s, p->precision, best, s->kick_grid);
+        // (one block when there is nothing to pull anything)
+        s->kick_grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)s->items.size(), (int64_t)s->nsm * graph_blocks(best)));
         snprintf(s->kick_desc, sizeof(s->kick_desc), "%s, grid %d, %zu items, %d j-chunks (system 0)%s",
                  kick_variant_name(p->precision, best), s->kick_grid, s->items.size(), s->sys[0].nchunk,
                  force ? ", forced" : (best_ms >= 0 ? ", autotuned" : ""));
@@ -646,7 +696,7 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
     {
         // warps a position takes in the row sums: eight rows a warp, at most eight warps
         int32_t maxc = 1;
-        for (auto& si : s->sys) maxc = std::max(maxc, si.nchunk);
+        for (auto& si : s->sys) maxc = std::max({maxc, si.nchunk, si.nchunk_small});
         d.rows_g = 1;
         while (d.rows_g < 8 && d.rows_g * 8 < maxc) d.rows_g *= 2;
     }

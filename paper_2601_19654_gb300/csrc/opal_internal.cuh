@@ -21,6 +21,7 @@ constexpr int64_t kHugeWaitNs = 4000000000;   // the whole-GPU encounter kernel'
 constexpr int kHugeAbortDetail = 2999999;      // status detail of its barrier aborts: this, or this + 1 + group
 constexpr int kKickJTile = 256;
 constexpr int kKickBox = 128;      // positions per tile box of the kick's sorted copies     // j-bodies the kick stages in shared memory at a time
+constexpr int kKickSuperMax = 64;  // tiles of a super-tile of the FP64 kick at most
 constexpr int kBsManyGroups = 608;  // above this many groups a step integrates them packed, lane per member
 constexpr int kBucketDiv = 4;       // body slots per bucket of the spatial sort (cap / 4 buckets a system)
 constexpr int kBsOut = 9;           // doubles per member slot of the BS side buffer: x, V, m, R, alive
@@ -130,10 +131,11 @@ struct SysInfo {
     int64_t nseg;     // cap / kSeg
     int64_t slot0;    // first row of the kick's partial-acceleration buffer
     int32_t nchunk;   // j-chunks of the kick for this system
-    int32_t pad;
+    int32_t nchunk_small;   // the same for the small bodies (FP64 form; else nchunk)
 };
 
-// One unit of kick work: an i-tile against a j-range of the same system.
+// One unit of kick work: an i-tile against a j-range of the same system (FP64
+// form: two super-tiles of istep bodies, or with istep 0 small bodies against big ones).
 struct KickItem {
     int32_t sys;
     int32_t chunk;    // index of the j-range within the system (the partial row it writes)
@@ -191,6 +193,7 @@ struct Dev {
     float *ks_x, *ks_y, *ks_z, *ks_m;
     float4* ks_lo;
     float* ks_rc;
+    int kick_smem = 0;   // dynamic shared memory of the kick (FP64 form: the j side's sums)
     int rows_g = 8;  // warps a position takes in k_kick_rows (1, 2, 4 or 8: eight rows a warp)
     unsigned long long* timeline = nullptr;   // [kTlCount][2] (timeline builds only)
     double* ksum;    // [3 ntot]: each body's kick partial rows summed (by k_kick_rows), by body index
@@ -666,7 +669,6 @@ const char* kick_variant_name(int precision, int variant);
 int kick_occupancy(int precision, int variant);
 int kick_threads(int precision, int variant);      // threads a block of variant v
 int kick_itile(int precision, int variant);   // i-bodies per i-tile (a divisor of kPad)
-bool kick_jmajor(int precision, int variant); // items: one j-tile against a run of i-tiles (else an i-tile against j-tiles)
 void launch_kick_stage(const Dev& d, int precision, cudaStream_t s);   // the sorted copies the mixed kick reads
 void launch_kick_rows(const Dev& d, cudaStream_t s);   // after every kick: its partial rows summed a body
 void launch_close(const Dev& d, cudaStream_t s);

@@ -712,19 +712,13 @@ __global__ void __launch_bounds__(256) k_group_order(Dev d) {
             if (n <= d.hb.cap) d.ghuge[atomicAdd(&d.ctl->nhuge, 1)] = g;
             else set_status(d.ctl, kEoverflow, 2000000 + g);
         } else if (threadIdx.x == 0) {
-            if (ng > kBsManyGroups) {
-                // many groups: up to 16 members to the packed kernel's class lists, larger
-                // ones straight to the lockstep kernels
-                if (n <= 16) {
-                    const int c = n <= 2 ? 0 : (n <= 4 ? 1 : (n <= 8 ? 2 : 3));
-                    d.gcls[c * d.gcap + atomicAdd(&d.ctl->ncls[c], 1)] = g;
-                } else {
-                    const int q = atomicAdd(&d.ctl->nhard, 1);
-                    if (q < d.gcap) d.ghard[q] = g;
-                    else set_status(d.ctl, kEoverflow, -7);
-                }
-            } else if (n > 4) {
-                d.glarge[atomicAdd(&d.ctl->nlarge, 1)] = g;
+            // more than four members: the larger groups' lockstep kernels; many groups:
+            // the others to the packed kernel's class lists
+            if (n > 16) d.glarge[atomicAdd(&d.ctl->nlarge, 1)] = g;
+            else if (n > 4) d.gmid[atomicAdd(&d.ctl->nmid, 1)] = g;
+            else if (ng > kBsManyGroups) {
+                const int c = n <= 2 ? 0 : 1;
+                d.gcls[c * d.gcap + atomicAdd(&d.ctl->ncls[c], 1)] = g;
             }
         }
         for (int k = threadIdx.x; k < n; k += blockDim.x) {

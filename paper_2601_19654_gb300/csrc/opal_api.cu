@@ -71,9 +71,9 @@ struct opal_sim {
     cudaStream_t stream = nullptr;
     cudaStream_t side = nullptr;             // the kick's branch of the step graph
     cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
-    cudaStream_t side2 = nullptr;            // the large-group BS kernels' branch (in order)
-    cudaStream_t side3 = nullptr;            // the same beside the kick, one priority lower
-    cudaEvent_t fork2_ev = nullptr, join2_ev = nullptr;
+    cudaStream_t side2 = nullptr;            // the 5-16-member groups' branch (in order)
+    cudaStream_t side3 = nullptr;            // the larger groups'; beside the kick both, one priority lower
+    cudaEvent_t fork2_ev = nullptr, join2_ev = nullptr, join3_ev = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     std::vector<SysInfo> sys;
@@ -391,6 +391,7 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
     CKF(cudaStreamCreateWithPriority(&s->side3, cudaStreamNonBlocking, prio_mid));
     CKF(cudaEventCreateWithFlags(&s->fork2_ev, cudaEventDisableTiming));
     CKF(cudaEventCreateWithFlags(&s->join2_ev, cudaEventDisableTiming));
+    CKF(cudaEventCreateWithFlags(&s->join3_ev, cudaEventDisableTiming));
     CKF(bs_setup());
 
     // parameters
@@ -504,9 +505,10 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
     TRYF(dalloc(s, &d.flag, d.flag_cap));
     TRYF(dalloc(s, &d.members, 2 * d.flag_cap + 2));
     TRYF(dalloc(s, &d.goff, 2 * d.flag_cap + 2));
+    TRYF(dalloc(s, &d.gmid, 2 * d.flag_cap + 2));
     TRYF(dalloc(s, &d.glarge, 2 * d.flag_cap + 2));
     d.gcap = std::min<int64_t>(d.flag_cap + 1, N / 2 + 1);   // a group has two members at least
-    TRYF(dalloc(s, &d.gcls, 4 * d.gcap));
+    TRYF(dalloc(s, &d.gcls, 2 * d.gcap));
     TRYF(dalloc(s, &d.ghard, d.gcap));
     TRYF(dalloc(s, &d.ghuge, d.gcap));
     {
@@ -761,10 +763,9 @@ void launch_stage(opal_sim* s, int k, cudaStream_t st) {
         case 3: launch_confirm(d, s->confirm_grid, st); break;
         case 4: launch_group(d, s->nsm, st); break;
         case kStageBs:
-            // the lockstep kernels on parallel branches (one stream when profiling)
-            launch_bs_packed(d, s->nsm, st);
-            note_launch(s, launch_bs_lockstep(d, s->nsm, st, g_prof ? st : s->side2, s->fork2_ev, s->join2_ev,
-                                              false));
+            // the encounter kernels on parallel branches (one stream when profiling)
+            note_launch(s, launch_bs(d, s->nsm, st, g_prof ? st : s->side2, g_prof ? st : s->side3, s->fork2_ev, s->join2_ev,
+                                     s->join3_ev, false));
             break;
         case kStageKick:
             launch_kick_stage(d, d.p.precision, st);
@@ -837,7 +838,8 @@ opal_status capture_graph(opal_sim* s) {
             CK(cudaStreamWaitEvent(s->side, s->fork_ev, 0));
             launch_stage(s, kStageKick, s->side);
             CK(cudaEventRecord(s->join_ev, s->side));
-            note_launch(s, launch_bs_lockstep(s->d, s->nsm, s->stream, s->side3, s->fork2_ev, s->join2_ev, true));
+            note_launch(s, launch_bs(s->d, s->nsm, s->stream, s->side3, s->side3, s->fork2_ev, s->join2_ev,
+                                     s->join3_ev, true));
             CK(cudaStreamWaitEvent(s->stream, s->join_ev, 0));
             continue;
         }
@@ -1174,6 +1176,7 @@ void opal_destroy(opal_sim* s) {
     if (s->side3) cudaStreamDestroy(s->side3);
     if (s->fork2_ev) cudaEventDestroy(s->fork2_ev);
     if (s->join2_ev) cudaEventDestroy(s->join2_ev);
+    if (s->join3_ev) cudaEventDestroy(s->join3_ev);
     delete s;
 }
 
@@ -1352,14 +1355,13 @@ opal_status opal_debug_bs_group(opal_sim* s, const double* x0, const double* V0,
     c.ninvolved = (int)n;
     if (n > 4) {
         int zero = 0;
-        c.nlarge = 1;
-        CK(cudaMemcpy(d.glarge, &zero, sizeof(int), cudaMemcpyHostToDevice));
+        (n > 16 ? c.nlarge : c.nmid) = 1;
+        CK(cudaMemcpy(n > 16 ? d.glarge : d.gmid, &zero, sizeof(int), cudaMemcpyHostToDevice));
     }
     CK(cudaMemcpy(d.ctl, &c, sizeof(Ctl), cudaMemcpyHostToDevice));
     CK(cudaMemsetAsync(d.mlo, 0x7f, d.nsys * sizeof(int), s->stream));
     CK(cudaMemsetAsync(d.mhi, 0, d.nsys * sizeof(int), s->stream));
-    launch_bs_packed(d, s->nsm, s->stream);
-    CK(launch_bs_lockstep(d, s->nsm, s->stream, s->stream, nullptr, nullptr, false));
+    CK(launch_bs(d, s->nsm, s->stream, s->stream, s->stream, nullptr, nullptr, nullptr, false));
     launch_bs_apply(d, s->nsm, s->stream);   // puts the result into the state
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(s->stream));
@@ -1403,7 +1405,7 @@ const char* opal_timeline_name(int32_t id) {
     static const char* names[kTlCount] = {
         "k_step_reset", "k_open", "k_sort_count", "k_sort_prefix", "k_sort_scatter", "k_sort_order",
         "k_tile_box", "k_tile_cull", "k_scan_tiles", "k_chord", "k_confirm", "k_group_link", "k_group_count",
-        "k_group_offsets", "k_group_place", "k_group_order", "k_bs_packed", "k_bs_ws", "k_bs<256>", "k_bs<512>",
+        "k_group_offsets", "k_group_place", "k_group_order", "k_bs_packed", "k_bs_ws", "k_bs_ws<4>", "k_bs",
         "k_bs_huge", "k_kick_stage", "k_kick", "k_kick_rows", "k_kick_apply", "k_kick_fix", "k_close",
         "k_finish"};
     return id >= 0 && id < kTlCount ? names[id] : nullptr;

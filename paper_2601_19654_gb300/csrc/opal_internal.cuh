@@ -22,7 +22,9 @@ constexpr int kHugeAbortDetail = 2999999;      // status detail of its barrier a
 constexpr int kKickJTile = 256;
 constexpr int kKickBox = 128;      // positions per tile box of the kick's sorted copies     // j-bodies the kick stages in shared memory at a time
 constexpr int kKickSuperMax = 64;  // tiles of a super-tile of the FP64 kick at most
-constexpr int kBsManyGroups = 608;  // above this many groups a step integrates them packed, lane per member
+constexpr int kBsManyGroups = 4864;  // above this many groups a step integrates those of up to 4 members packed, lane per member
+constexpr int kBsSoloGroups = 608;  // above this many groups the small-group kernel makes one attempt at a time
+constexpr int kBsSoloMid = 76;      // the same for groups of 5-16 members, above this many of them
 constexpr int kBucketDiv = 4;       // body slots per bucket of the spatial sort (cap / 4 buckets a system)
 constexpr int kBsOut = 9;           // doubles per member slot of the BS side buffer: x, V, m, R, alive
 constexpr int kFixParts = 4;        // the kick's correction after the encounters: member ranges per body
@@ -55,11 +57,11 @@ struct Ctl {
     int nacc, nej;       // bodies accreted and ejected at the end of the step (this step)
     int nmerge;          // mergers (this step)
     int kepler_max;      // largest drift iteration count (this step)
-    int nlarge;          // groups too large for one warp (this step)
-    int ncls[4];         // groups of 2, 3-4, 5-8, 9-16 members (this step)
-    int qcls[4];         // how far the packed encounter kernel has taken each list (this step)
-    int nhard;           // groups left to the lockstep kernels when groups are many (this step)
-    int qlock[3];        // queues of the lockstep kernels: up to 4, 32, 64 members (this step)
+    int nmid, nlarge;    // groups of 5-16 and of 17-64 members (this step)
+    int ncls[2];         // groups of 2 and of 3-4 members when groups are many (this step)
+    int qcls[2];         // how far the packed encounter kernel has taken each list (this step)
+    int nhard;           // groups the packed kernel leaves to the lockstep kernel (this step)
+    int qlock[3];        // queues of the lockstep kernels: up to 4, 16, 64 members (this step)
     int nhuge;           // groups of more than 64 members (this step)
     int ntov;            // tile pairs whose boxes overlap (this step)
     unsigned long long nsub;  // BS substeps (this step)
@@ -232,9 +234,9 @@ struct Dev {
     int32_t* label;                     // per body; -1 when not in a group
     int32_t* members;                   // group members, grouped, ascending
     int32_t* goff;                      // [ngroups + 1] member offsets
-    int32_t* glarge;                    // groups of more than 4 members
-    int32_t* gcls;                      // [4][gcap]: groups by size class (2, 4, 8, 16 members at most)
-    int32_t* ghard;                     // [gcap]: groups for the lockstep kernels when groups are many
+    int32_t *gmid, *glarge;             // groups of 5-16 and of 17-64 members
+    int32_t* gcls;                      // [2][gcap]: groups by size class (2 and 4 members at most)
+    int32_t* ghard;                     // [gcap]: groups the packed kernel leaves to the lockstep kernel
     int32_t* ghuge;                     // [gcap]: groups of more than 64 members
     HugeBuf hb;                         // working arrays of the whole-GPU encounter kernel
     HugeCtl* hctl;
@@ -375,10 +377,23 @@ __device__ __forceinline__ bool le_zero(double a) { return __double_as_longlong(
 __device__ __forceinline__ double mutual_factor(double gm_ri3, double y, int form) {
     if (__double_as_longlong(y) <= 0) return gm_ri3;   // y <= 0: K = 0
     if (form == 0) {
-        const double u = 1.0 - y;
+        const double u = __dadd_rn(1.0, -y);   // (not contracted with y's product, wherever this is inlined)
         return (gm_ri3 * (u * u)) / fma(2.0 * y, -u, 1.0);   // 2y^2 - 2y + 1 = 1 - 2y(1 - y)
     }
     return gm_ri3 * (1.0 - y * y * y * (10.0 - 15.0 * y + 6.0 * y * y));
+}
+
+// v rounded toward zero to a float, on the integer units: a warp's F2F from
+// FP64 holds the scheduler's FP64 unit for about 70 cycles (measured), as an
+// FP64 operation does, where this is about eight integer instructions.  Below
+// the normal floats 0, above them an infinity (a NaN becomes one too).
+__device__ __forceinline__ float trunc_f(double v) {
+    const int hi = __double2hiint(v), lo = __double2loint(v);
+    const int e = (hi >> 20) & 0x7ff;
+    unsigned f = (__funnelshift_l((unsigned)lo, (unsigned)hi, 3) - (896u << 23)) & 0x7fffffffu;
+    if (e < 897) f = 0u;
+    if (e > 1150) f = 0x7f800000u;
+    return __uint_as_float(f | ((unsigned)hi & 0x80000000u));
 }
 
 // Changeover weight K(r; rc): the rational form y^2/(2y^2-2y+1) or the
@@ -615,7 +630,7 @@ inline void prof_mark(const char* name) {
 enum TimelineId {
     kTlReset, kTlOpen, kTlSortCount, kTlSortPrefix, kTlSortScatter, kTlSortOrder, kTlTileBox, kTlTileCull,
     kTlScanTiles, kTlChord, kTlConfirm, kTlGroupLink, kTlGroupCount, kTlGroupOffsets, kTlGroupPlace,
-    kTlGroupOrder, kTlBsPacked, kTlBsWs, kTlBs256, kTlBs512, kTlBsHuge, kTlKickStage, kTlKick, kTlKickRows,
+    kTlGroupOrder, kTlBsPacked, kTlBsWs, kTlBs16, kTlBs64, kTlBsHuge, kTlKickStage, kTlKick, kTlKickRows,
     kTlApply, kTlFix, kTlClose, kTlFinish, kTlCount
 };
 #ifdef OPAL_TIMELINE
@@ -656,8 +671,8 @@ void launch_confirm(const Dev& d, int grid, cudaStream_t s);
 void launch_group(const Dev& d, int nsm, cudaStream_t s);
 cudaError_t bs_setup();   // dynamic shared memory of the BS kernels
 void launch_bs_packed(const Dev& d, int nsm, cudaStream_t s);
-cudaError_t launch_bs_lockstep(const Dev& d, int nsm, cudaStream_t s, cudaStream_t s2, cudaEvent_t fork, cudaEvent_t join,
-                        bool small_first);
+cudaError_t launch_bs(const Dev& d, int nsm, cudaStream_t s, cudaStream_t s2, cudaStream_t s3, cudaEvent_t fork,
+                      cudaEvent_t join, cudaEvent_t join3, bool beside);
 void launch_kick(const Dev& d, const KickItem* items, int64_t nitems, int grid, int precision, int variant,
                  cudaStream_t s);
 // after the BS: apply its results; fix the kick's rows when it ran beside the BS

@@ -29,6 +29,8 @@
 
 #include <type_traits>
 
+#include <algorithm>
+
 #include "opal_internal.cuh"
 
 namespace opal {
@@ -672,9 +674,9 @@ __global__ void __launch_bounds__(32 * kPkWarps) k_bs_packed(Dev d) {
 // members, k_bs_ws<4> five to sixteen.  The attempts (step sizes H, H/2, H/4,
 // H/8, or H and H/2) are the blocks of a cluster; when every one is rejected
 // the next round tries the following halvings, so the sizes tried and
-// accepted are those of the sequential scheme.  Inside a block four roles of R
-// warps each (R = 1 up to four members, else a quarter of the members) share
-// the work of a round, since a warp's FP64 instruction holds its scheduler's
+// accepted are those of the sequential scheme.  Inside a block four roles share
+// the work of a round (a warp each up to four members; else R warps, a quarter of the
+// members, for roles 0 and 3 and half of the other warps each for roles 1 and 2), since a warp's FP64 instruction holds its scheduler's
 // FP64 unit for 64 cycles whatever its dependences, so that what shortens a
 // round is fewer instructions on the warp that waits:
 //   role 0 keeps each (sequence, member) state and takes the midpoint steps;
@@ -1382,6 +1384,7 @@ void launch_bs_packed(const Dev& d, int nsm, cudaStream_t s) {
     // one block of four warps an SM, one a scheduler (a scheduler's FP64 unit takes 64 cycles a warp
     // instruction, so a second warp there would wait for the first): the ensemble's first attempts
     // 2.6 ms with two warps, 1.52 with four, 1.45 with eight, a few hundred groups 0.41, 0.42 and 0.46
+    if (d.ntot / 2 <= kBsManyGroups) return;   // (a group has two members at least)
     k_bs_packed<<<nsm, 32 * kPkWarps, kPkWarps * sizeof(PkWarp), s>>>(d);
     prof_mark("bs: many groups, packed");
 }
@@ -1401,6 +1404,7 @@ void launch_bs_packed(const Dev& d, int nsm, cudaStream_t s) {
 cudaError_t launch_bs(const Dev& d, int nsm, cudaStream_t s, cudaStream_t s2, cudaStream_t s3, cudaEvent_t fork,
                       cudaEvent_t join, cudaEvent_t join3, bool beside) {
     cudaError_t err = cudaSuccess;   // the first failed launch, if any (the cluster and cooperative ones)
+    if (d.nmax <= 4) s2 = s3 = s;    // (no larger groups)
     if (s2 != s) {
         cudaEventRecord(fork, s);
         cudaStreamWaitEvent(s2, fork, 0);
@@ -1422,11 +1426,18 @@ cudaError_t launch_bs(const Dev& d, int nsm, cudaStream_t s, cudaStream_t s2, cu
         const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, d);
         if (err == cudaSuccess) err = e;
     };
+    // no more blocks than groups of at least so many members can form
+    const int64_t bodies = (int64_t)d.nmax * d.nsys;
+    auto room = [&](int least, int64_t blocks) { return (int)std::min<int64_t>(blocks, std::max<int64_t>(1, bodies / least)); };
     auto larger = [&] {
-        clusters(k_bs_ws<4, kWsAttemptsMid>, sizeof(WsSh<4>), kWsAttemptsMid, nsm, 512, s2);
+        if (d.nmax <= 4) return;   // (kernels whose groups cannot form are left out)
+        clusters(k_bs_ws<4, kWsAttemptsMid>, sizeof(WsSh<4>), kWsAttemptsMid,
+                 kWsAttemptsMid * room(5, nsm / kWsAttemptsMid), 512, s2);
         if (s2 == s) prof_mark("bs: groups of 5-16");
-        k_bs<<<nsm, kBsThreads, sizeof(BsSh), s3>>>(d);
+        if (d.nmax <= 16) return;
+        k_bs<<<room(17, nsm), kBsThreads, sizeof(BsSh), s3>>>(d);
         if (s2 == s) prof_mark("bs: groups of 17-64");
+        if (d.nmax <= 64) return;
         const cudaError_t e = launch_bs_huge(d, nsm, s3);
         if (err == cudaSuccess) err = e;
     };
@@ -1435,8 +1446,10 @@ cudaError_t launch_bs(const Dev& d, int nsm, cudaStream_t s, cudaStream_t s2, cu
         launch_bs_packed(d, nsm, s);
     }
     // groups of up to 4 members: clusters of two or four blocks, one attempt each
-    if (beside) clusters(k_bs_ws<1, kWsAttemptsBeside>, sizeof(WsSh<1>), kWsAttemptsBeside, 2 * kWsAttemptsBeside * nsm, 128, s);
-    else clusters(k_bs_ws<1, kWsAttemptsAlone>, sizeof(WsSh<1>), kWsAttemptsAlone, 2 * kWsAttemptsAlone * nsm, 128, s);
+    if (beside) clusters(k_bs_ws<1, kWsAttemptsBeside>, sizeof(WsSh<1>), kWsAttemptsBeside,
+                         kWsAttemptsBeside * room(2, 2 * nsm), 128, s);
+    else clusters(k_bs_ws<1, kWsAttemptsAlone>, sizeof(WsSh<1>), kWsAttemptsAlone,
+                  kWsAttemptsAlone * room(2, 2 * nsm), 128, s);
     prof_mark("bs: groups <= 4");
     if (beside) larger();
     if (s2 != s) {

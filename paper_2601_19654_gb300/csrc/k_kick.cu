@@ -952,6 +952,110 @@ __global__ void __launch_bounds__(kFixThreads) k_kick_fix(Dev d, int nbody_block
     }
 }
 
+// The mixed kick of a small system (kSmallBodies bodies at most), in order
+// after the encounters: a warp a body, its lanes the big bodies in turn, from
+// the float copies as they lie (nothing sorted or staged, no partial rows); one
+// more block sums the closing jump's momentum beside it.  It is latency that
+// counts at these sizes: 3 us in place of 16 for staging, kick, rows and the fix's momentum
+// with 10 bodies, 5 in place of 80 with 1001 (32 tiles held 32 SMs).
+// Precision: every pair has the lo parts (the tiled kick adds them within 2 (rc_i +
+// rc_max) only) and a reciprocal square root refined by a Newton step, the
+// changeover where the pair is within the larger critical radius; eight terms
+// at a time are folded into a lane's hi/lo pair and the lanes are added as float pairs.
+constexpr int kSmallKickThreads = 256;
+__global__ void __launch_bounds__(kSmallKickThreads) k_kick_small(Dev d, int nblk) {
+    OPAL_TIMELINE_SCOPE(kTlKick);
+    if (d.ctl->status || (d.gated && !d.ctl->reprime)) return;
+    const SysInfo si = d.sys[0];
+    const int tid = threadIdx.x, lane = tid & 31;
+    if ((int)blockIdx.x == nblk) {   // momentum of the state after the encounters
+        __shared__ double red[3][kSmallKickThreads];
+        double px = 0.0, py = 0.0, pz = 0.0;
+        for (int64_t b = si.off + tid; b < si.off + si.n; b += kSmallKickThreads) {
+            const double m = d.alive[b] ? d.m[b] : 0.0;
+            px += m * d.vx[b];
+            py += m * d.vy[b];
+            pz += m * d.vz[b];
+        }
+        red[0][tid] = px;
+        red[1][tid] = py;
+        red[2][tid] = pz;
+        __syncthreads();
+        for (int w = kSmallKickThreads / 2; w >= 1; w >>= 1) {
+            if (tid < w)
+                for (int c = 0; c < 3; c++) red[c][tid] += red[c][tid + w];
+            __syncthreads();
+        }
+        if (tid < 3) {
+            d.Ptot[3 * d.nsys + tid] = red[tid][0];
+            d.Pjump[3 * d.nsys + tid] = 0.5 * d.p.dt * red[tid][0] / d.M0s[0];
+        }
+        return;
+    }
+    const int64_t k = (int64_t)blockIdx.x * (kSmallKickThreads / 32) + (tid >> 5);
+    if (k >= si.n) return;   // (whole warps; no barrier follows)
+    const int64_t i = si.off + k;
+    const float4 hi = d.kh[i], li = d.kl[i];
+    const float rci = d.rcf[i];
+    const int form = d.p.changeover;
+    const int64_t jend = si.off + si.nb;
+    float2 sx = make_float2(0.0f, 0.0f), sy = sx, sz = sx;
+    for (int64_t j0 = si.off + lane; j0 < jend; j0 += 8 * 32) {
+        float4 hj[8], lj[8];
+        float rcj[8];
+#pragma unroll
+        for (int u = 0; u < 8; u++) {
+            const int64_t j = j0 + 32 * u;
+            const bool in = j < jend && j != i;
+            hj[u] = in ? d.kh[j] : make_float4(kFar, kFar, kFar, 0.0f);
+            lj[u] = in ? d.kl[j] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            rcj[u] = in ? d.rcf[j] : 0.0f;
+        }
+        float tx = 0.0f, ty = 0.0f, tz = 0.0f;
+#pragma unroll
+        for (int u = 0; u < 8; u++) {
+            const float dx = (hj[u].x - hi.x) + (lj[u].x - li.x), dy = (hj[u].y - hi.y) + (lj[u].y - li.y),
+                        dz = (hj[u].z - hi.z) + (lj[u].z - li.z);
+            const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+            const float rcij = fmaxf(rci, rcj[u]);
+            float s;
+            if (r2 < fmaxf(1.0001f * (rcij * rcij), 1e-30f)) {   // (the margin covers the roundings)
+                s = 0.0f;
+                if (r2 > 0.0f) {
+                    const float r = sqrtf(r2);
+                    s = hj[u].w * changeover_f(r, rcij, form) / (r2 * r);
+                }
+            } else {
+                float y = rsqrt_approx(r2);
+                y = fmaf(0.5f * y, fmaf(-(r2 * y), y, 1.0f), y);
+                s = (hj[u].w * y) * (y * y);
+            }
+            tx = fmaf(s, dx, tx);
+            ty = fmaf(s, dy, ty);
+            tz = fmaf(s, dz, tz);
+        }
+        fold(sx.x, sx.y, tx);
+        fold(sy.x, sy.y, ty);
+        fold(sz.x, sz.y, tz);
+    }
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {   // (the sum of two float pairs does not depend on their order)
+        sx = ff_add(sx, make_float2(__shfl_xor_sync(0xffffffffu, sx.x, o), __shfl_xor_sync(0xffffffffu, sx.y, o)));
+        sy = ff_add(sy, make_float2(__shfl_xor_sync(0xffffffffu, sy.x, o), __shfl_xor_sync(0xffffffffu, sy.y, o)));
+        sz = ff_add(sz, make_float2(__shfl_xor_sync(0xffffffffu, sz.x, o), __shfl_xor_sync(0xffffffffu, sz.y, o)));
+    }
+    if (lane < 3) {
+        const float2 a = lane == 0 ? sx : (lane == 1 ? sy : sz);
+        d.ksum[3 * i + lane] = (double)a.x + (double)a.y;
+    }
+}
+
+void launch_kick_small(const Dev& d, cudaStream_t s) {
+    const int nblk = (d.nmax + kSmallKickThreads / 32 - 1) / (kSmallKickThreads / 32);
+    k_kick_small<<<nblk + (d.gated ? 0 : 1), kSmallKickThreads, 0, s>>>(d, nblk);
+    prof_mark("kick");
+}
+
 void launch_bs_apply(const Dev& d, int nsm, cudaStream_t s) {
     k_kick_apply<<<nsm, 256, 0, s>>>(d);
     prof_mark("apply BS results");

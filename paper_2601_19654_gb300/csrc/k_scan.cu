@@ -492,6 +492,35 @@ __device__ double interval_min2(double T, int k, const double* d0, const double*
     return fmax(D, 0.0);
 }
 
+// Stage 3 of one pair by 16 lanes (sub: the lane's place among them, half: their
+// mask); live: there is a pair.  The pair is flagged when its minimum separation
+// is within the critical distance, and both ends become members.
+__device__ __forceinline__ void confirm_pair(const Dev& d, int2 pr, bool live, int sub, unsigned half) {
+    double D = HUGE_VAL, rcij = 0.0;
+    if (live) {
+        const int i = pr.x, j = pr.y;
+        double d0[3] = {d.x0[j] - d.x0[i], d.y0[j] - d.y0[i], d.z0[j] - d.z0[i]};
+        double u0[3] = {d.vx0[j] - d.vx0[i], d.vy0[j] - d.vy0[i], d.vz0[j] - d.vz0[i]};
+        double d1[3] = {d.x[j] - d.x[i], d.y[j] - d.y[i], d.z[j] - d.z[i]};
+        double u1[3] = {d.vx[j] - d.vx[i], d.vy[j] - d.vy[i], d.vz[j] - d.vz[i]};
+        rcij = fmax(d.rc[i], d.rc[j]);
+        D = fmin(dot3p(d0, d0), dot3p(d1, d1));
+        D = fmin(D, interval_min2(d.p.dt, sub, d0, u0, d1, u1));
+    }
+#pragma unroll
+    for (int o = 8; o >= 1; o >>= 1) D = fmin(D, __shfl_xor_sync(half, D, o));
+    if (live && sub == 0 && D <= rcij * rcij) {
+        int idx = atomicAdd(&d.ctl->nflag, 1);
+        if (idx < d.flag_cap) {
+            d.flag[idx] = pr;
+            d.label[pr.x] = pr.x;   // both ends become members (their own union-find roots)
+            d.label[pr.y] = pr.y;
+        } else {
+            set_status(d.ctl, kEoverflow, -2);
+        }
+    }
+}
+
 __global__ void __launch_bounds__(256) k_confirm(Dev d) {
     OPAL_TIMELINE_SCOPE(kTlConfirm);
     if (d.ctl->status) return;
@@ -500,7 +529,6 @@ __global__ void __launch_bounds__(256) k_confirm(Dev d) {
         if (blockIdx.x == 0 && threadIdx.x == 0) set_status(d.ctl, kEoverflow, -1);
         return;
     }
-    const double T = d.p.dt;
     const int lane = threadIdx.x & 31, sub = lane & 15;
     const unsigned half = 0xffffu << (lane & 16);
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -514,29 +542,7 @@ __global__ void __launch_bounds__(256) k_confirm(Dev d) {
             pr = d.cand[k];
             live = d.alive[pr.x] && d.alive[pr.y];
         }
-        double D = HUGE_VAL, rcij = 0.0;
-        if (live) {
-            const int i = pr.x, j = pr.y;
-            double d0[3] = {d.x0[j] - d.x0[i], d.y0[j] - d.y0[i], d.z0[j] - d.z0[i]};
-            double u0[3] = {d.vx0[j] - d.vx0[i], d.vy0[j] - d.vy0[i], d.vz0[j] - d.vz0[i]};
-            double d1[3] = {d.x[j] - d.x[i], d.y[j] - d.y[i], d.z[j] - d.z[i]};
-            double u1[3] = {d.vx[j] - d.vx[i], d.vy[j] - d.vy[i], d.vz[j] - d.vz[i]};
-            rcij = fmax(d.rc[i], d.rc[j]);
-            D = fmin(dot3p(d0, d0), dot3p(d1, d1));
-            D = fmin(D, interval_min2(T, sub, d0, u0, d1, u1));
-        }
-#pragma unroll
-        for (int o = 8; o >= 1; o >>= 1) D = fmin(D, __shfl_xor_sync(half, D, o));
-        if (live && sub == 0 && D <= rcij * rcij) {
-            int idx = atomicAdd(&d.ctl->nflag, 1);
-            if (idx < d.flag_cap) {
-                d.flag[idx] = pr;
-                d.label[pr.x] = pr.x;   // both ends become members (their own union-find roots)
-                d.label[pr.y] = pr.y;
-            } else {
-                set_status(d.ctl, kEoverflow, -2);
-            }
-        }
+        confirm_pair(d, pr, live, sub, half);
     }
 }
 
@@ -765,6 +771,295 @@ __global__ void __launch_bounds__(256) k_group_order(Dev d) {
     }
 }
 
+// ---------------------------------------------------------------- small systems
+// The scan and the groups of one small system in one kernel.  (One block for the groups
+// of larger systems was slower than the five kernels: 12 against 9 us at 5003 bodies, 30
+// against 10 at 16384; in shared memory, up to kSmallBodies bodies, it takes 5 in place of 9.)
+
+// exclusive scan over the block of (members, groups) packed in a long long
+template <int NT>
+__device__ __forceinline__ long long block_excl(long long sum, long long* warp_sum, long long& total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    long long x = sum;
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) warp_sum[warp] = x;
+    __syncthreads();
+    long long before = 0;
+    total = 0;
+#pragma unroll
+    for (int w = 0; w < NT / 32; w++) {
+        const long long ws = warp_sum[w];
+        if (w < warp) before += ws;
+        total += ws;
+    }
+    __syncthreads();
+    return before + x - sum;
+}
+
+// ranges ascending, and the groups' lists: a thread a group of up to eight members, the
+// block the larger ones one after another (v: kSmallSlots ints)
+template <int NT>
+__device__ void group_order_block(const Dev& d, int ng, int* v) {
+    const int tid = threadIdx.x;
+    for (int g = tid; g < ng; g += NT) {
+        const int m0 = d.goff[g], n = d.goff[g + 1] - m0;
+        if (n > 64) {
+            if (n <= d.hb.cap) d.ghuge[atomicAdd(&d.ctl->nhuge, 1)] = g;
+            else set_status(d.ctl, kEoverflow, 2000000 + g);
+        } else if (n > 16) {
+            d.glarge[atomicAdd(&d.ctl->nlarge, 1)] = g;
+        } else if (n > 4) {
+            d.gmid[atomicAdd(&d.ctl->nmid, 1)] = g;
+        }   // (too few groups for the packed kernel's lists)
+        if (n > 8) continue;
+        int m[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) m[k] = k < n ? d.members[m0 + k] : 0x7fffffff;
+#pragma unroll
+        for (int r = 0; r < 8; r++)   // odd-even transposition: eight rounds sort eight
+#pragma unroll
+            for (int k = r & 1; k + 1 < 8; k += 2) {
+                const int lo = min(m[k], m[k + 1]), hi = max(m[k], m[k + 1]);
+                m[k] = lo;
+                m[k + 1] = hi;
+            }
+#pragma unroll
+        for (int k = 0; k < 8; k++)
+            if (k < n) d.members[m0 + k] = m[k];
+    }
+    __syncthreads();
+    for (int g = 0; g < ng; g++) {
+        const int m0 = d.goff[g], n = d.goff[g + 1] - m0;   // (the same for the whole block)
+        if (n <= 8) continue;
+        int np2 = 1;
+        while (np2 < n) np2 <<= 1;
+        __syncthreads();
+        for (int k = tid; k < np2; k += NT) v[k] = k < n ? d.members[m0 + k] : 0x7fffffff;
+        __syncthreads();
+        for (int size = 2; size <= np2; size <<= 1)
+            for (int stride = size >> 1; stride > 0; stride >>= 1) {
+                for (int k = tid; k < np2; k += NT) {
+                    const int q = k ^ stride;
+                    if (q > k) {
+                        const bool up = (k & size) == 0;
+                        const int x = v[k], y = v[q];
+                        if ((x > y) == up) {
+                            v[k] = y;
+                            v[q] = x;
+                        }
+                    }
+                }
+                __syncthreads();
+            }
+        for (int k = tid; k < n; k += NT) d.members[m0 + k] = v[k];
+    }
+}
+
+// a member into its group's range
+__device__ __forceinline__ void group_put(const Dev& d, int pos, int b) {
+    d.members[pos] = b;
+    d.undo[3 * (int64_t)pos + 2] = -1.0;
+    d.bsout[(int64_t)kBsOut * pos + 8] = -1.0;   // no result yet (the encounter kernels write one)
+}
+
+// root of x in shared memory; -1 if the walk runs past its bound
+__device__ __forceinline__ int uf_root_shared(int* parent, int x) {
+    volatile int* pv = parent;
+    for (int it = 0; it < kUfSteps; it++) {
+        const int p = pv[x];
+        if (p == x) return x;
+        const int gp = pv[p];
+        if (gp != p) atomicCAS(&parent[x], p, gp);
+        x = gp;
+    }
+    return -1;
+}
+
+// The groups of a small system, union-find and counts in shared memory: par and cnt
+// kSmallSlots ints each, par also for the members of a group being sorted.  What other
+// blocks have written is read past the L1 cache.
+constexpr int kSmallThreads = 256;
+constexpr int kSmallSlots = 2048;
+static_assert(kSmallBodies <= kSmallSlots, "a slot a body");
+__device__ void group_small(const Dev& d, int* par, int* cnt) {
+    constexpr int NT = kSmallThreads, PER = kSmallSlots / NT;
+    __shared__ long long warp_sum[NT / 32];
+    __shared__ int sstat;
+    const int tid = threadIdx.x;
+    if (tid == 0) sstat = __ldcg(&d.ctl->status);
+    __syncthreads();
+    const int nf = __ldcg(&d.ctl->nflag);
+    if (sstat || nf == 0) return;
+    if (nf > d.flag_cap) {
+        if (tid == 0) set_status(d.ctl, kEoverflow, -3);
+        return;
+    }
+#pragma unroll
+    for (int u = 0; u < PER; u++) {
+        par[u * NT + tid] = -1;
+        cnt[u * NT + tid] = 0;
+    }
+    __syncthreads();
+    for (int q = tid; q < nf; q += NT) {
+        const int2 pr = __ldcg(&d.flag[q]);
+        par[pr.x] = pr.x;
+        par[pr.y] = pr.y;
+    }
+    __syncthreads();
+    for (int q = tid; q < nf; q += NT) {
+        const int2 pr = __ldcg(&d.flag[q]);
+        bool done = false;
+        for (int it = 0; it < kUfSteps && !done; it++) {
+            const int ra = uf_root_shared(par, pr.x), rb = uf_root_shared(par, pr.y);
+            if (ra < 0 || rb < 0) break;
+            if (ra == rb) {
+                done = true;
+                break;
+            }
+            const int lo = min(ra, rb), hi = max(ra, rb);
+            done = atomicCAS(&par[hi], hi, lo) == hi;   // the larger root goes under the smaller
+        }
+        if (!done) set_status(d.ctl, kEoverflow, -5);
+    }
+    __syncthreads();
+    int root[PER], nbig = 0;
+    const int nb = (int)d.sys[0].nb;   // (one system, from body 0 on)
+#pragma unroll
+    for (int u = 0; u < PER; u++) {
+        const int b = u * NT + tid;
+        root[u] = par[b] < 0 ? -1 : uf_root_shared(par, b);
+        if (root[u] >= 0) {
+            atomicAdd(&cnt[root[u]], 1);
+            nbig += b < nb ? 1 : 0;
+        }
+    }
+    nbig = __reduce_add_sync(0xffffffffu, nbig);
+    if ((tid & 31) == 0 && nbig) atomicAdd(&d.ctl->ninv_big, nbig);
+    __syncthreads();
+    // scan in body order; par now holds each root's first member slot
+    int c[PER];
+    long long sum = 0, total;
+#pragma unroll
+    for (int u = 0; u < PER; u++) {
+        c[u] = cnt[tid * PER + u];
+        sum += (long long)c[u] + (c[u] > 0 ? (1LL << 32) : 0LL);
+    }
+    long long excl = block_excl<NT>(sum, warp_sum, total);
+#pragma unroll
+    for (int u = 0; u < PER; u++)
+        if (c[u] > 0) {
+            par[tid * PER + u] = (int)(excl & 0xffffffffLL);
+            d.goff[(int)(excl >> 32)] = (int)(excl & 0xffffffffLL);
+            excl += (long long)c[u] + (1LL << 32);
+        }
+    const int ng = (int)(total >> 32);
+    if (tid == 0) {
+        d.goff[ng] = (int)(total & 0xffffffffLL);
+        d.ctl->ngroups = ng;
+        d.ctl->ninvolved = (int)(total & 0xffffffffLL);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < PER; u++)
+        if (root[u] >= 0) group_put(d, par[root[u]] + atomicSub(&cnt[root[u]], 1) - 1, u * NT + tid);
+    __syncthreads();
+    group_order_block<NT>(d, ng, par);
+}
+
+// The whole scan of a small system (kSmallBodies bodies at most), unsorted: a
+// block a pair of 64-body tiles, all its pairs by the midpoint test, those that
+// pass by the chord bound, those by the exact minimum, in the block; the last
+// block to finish forms the groups.  One launch in place of fourteen, each a few
+// microseconds of latency at these sizes: alone 3 us in place of 21 with 10 bodies, 15 in
+// place of 38 with 1001 (and the launch gaps: a step of 10 bodies 87 to 43 us with the
+// small kick, of 1001 186 to 123).
+__global__ void __launch_bounds__(kSmallThreads) k_scan_small(Dev d, const PairTile* __restrict__ tiles, int ntiles,
+                                                              int group) {
+    OPAL_TIMELINE_SCOPE(kTlScanTiles);
+    __shared__ float4 sj[kSeg];
+    __shared__ __align__(16) unsigned short list[kSeg * kSeg];   // passing pairs: 64 i + j of the tile pair
+    __shared__ int par[kSmallSlots];
+    static_assert(sizeof(list) >= kSmallSlots * sizeof(int), "the list's room serves the counts of the groups");
+    __shared__ int count, kept, last, sstat;
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (tid == 0) sstat = d.ctl->status;
+    __syncthreads();   // (one reading for the whole block: another block may set it)
+    if (!sstat) {      // (otherwise the last block still has to be found)
+        for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
+            const PairTile tl = tiles[it];
+            const int64_t big_end = d.sys[tl.sys].off + d.sys[tl.sys].nb;   // ids below are big bodies
+            const int ii = tid & (kSeg - 1), part = tid / kSeg;             // four threads an i-body
+            const float4 ci = d.cen[tl.i0 + ii];
+            const bool ibig = tl.i0 + ii < big_end;
+            __syncthreads();
+            if (tid < kSeg) sj[tid] = d.cen[tl.j0 + tid];
+            if (tid == 0) count = kept = 0;
+            __syncthreads();
+            const bool diag = tl.i0 == tl.j0;
+#pragma unroll 4
+            for (int q = 0; q < kSeg / 4; q++) {
+                const int jj = part * (kSeg / 4) + q;
+                const float4 cj = sj[jj];
+                const float dx = cj.x - ci.x, dy = cj.y - ci.y, dz = cj.z - ci.z;
+                const float r2 = dx * dx + dy * dy + dz * dz, Ts = ci.w + cj.w;
+                // two small bodies never interact
+                if ((!diag || jj > ii) && r2 < Ts * Ts && (ibig || tl.j0 + jj < big_end))
+                    list[atomicAdd(&count, 1)] = (unsigned short)(ii * kSeg + jj);
+            }
+            __syncthreads();
+            const int n = count;
+            if (n == 0) continue;   // (the same for the whole block)
+            if (tid == 0) atomicAdd(&d.ctl->nnear, n);
+            // chord bound, the survivors compacted in place: a round's entries are read
+            // before any of its survivors is written, and those go below the entries read
+            for (int base = 0; base < n; base += kSmallThreads) {
+                const int k = base + tid;
+                bool pass = false;
+                int code = 0;
+                if (k < n) {
+                    code = list[k];
+                    const int64_t i = tl.i0 + code / kSeg, j = tl.j0 + code % kSeg;
+                    pass = d.alive[i] && d.alive[j] && chord_bound_passes(d, i, j, (float)d.p.dt);
+                }
+                __syncthreads();
+                const unsigned m = __ballot_sync(0xffffffffu, pass);
+                int at = 0;
+                if (lane == 0 && m) at = atomicAdd(&kept, __popc(m));
+                at = __shfl_sync(0xffffffffu, at, 0);
+                if (pass) list[at + __popc(m & ((1u << lane) - 1u))] = (unsigned short)code;
+                __syncthreads();
+            }
+            const int nc = kept;
+            if (tid == 0 && nc) atomicAdd(&d.ctl->ncand, nc);
+            const unsigned half = 0xffffu << (lane & 16);
+            for (int base = 0; base < nc; base += kSmallThreads / 16) {
+                const int k = base + tid / 16;
+                const bool live = k < nc;
+                const int code = live ? list[k] : 0;
+                confirm_pair(d, make_int2((int)tl.i0 + code / kSeg, (int)tl.j0 + code % kSeg), live, lane & 15, half);
+            }
+        }
+    }
+    // the last block out: everything the others flagged is there
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();
+        last = atomicAdd(&d.ctl->scan_done, 1) == (int)gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
+    if (tid == 0) {   // the list sizes of the general path bound this one too
+        if (__ldcg(&d.ctl->nnear) > d.near_cap) set_status(d.ctl, kEoverflow, -4);
+        else if (__ldcg(&d.ctl->ncand) > d.cand_cap) set_status(d.ctl, kEoverflow, -1);
+    }
+    __syncthreads();
+    if (group) group_small(d, par, reinterpret_cast<int*>(list));
+}
+
 void launch_sort_bodies(const Dev& d, cudaStream_t s) {
     const unsigned nb = (unsigned)(d.ntot / kBodyThreads);
     k_sort_count<<<nb, kBodyThreads, 0, s>>>(d);
@@ -792,6 +1087,11 @@ void launch_scan(const Dev& d, const PairTile* tiles, int64_t ntiles, int grid, 
 void launch_confirm(const Dev& d, int grid, cudaStream_t s) {
     k_confirm<<<grid, 256, 0, s>>>(d);
     prof_mark("confirm (FP64)");
+}
+
+void launch_scan_small(const Dev& d, const PairTile* tiles, int64_t ntiles, bool group, cudaStream_t s) {
+    k_scan_small<<<(unsigned)(ntiles < 1024 ? ntiles : 1024), kSmallThreads, 0, s>>>(d, tiles, (int)ntiles, group ? 1 : 0);
+    prof_mark("scan and groups of a small system");
 }
 
 void launch_group(const Dev& d, int nsm, cudaStream_t s) {

@@ -319,6 +319,16 @@ opal_status validate(const opal_params* p, char* err) {
     return OPAL_OK;
 }
 
+// One system of up to kSmallBodies bodies (padding included) whose step runs in
+// order: the scan and the groups in one kernel, unsorted, and in the mixed form
+// the kick a warp a body.  The all-pairs scan grows with the square: 15 us at 1001 bodies,
+// the sorted one's 38 there grow little (48 at 5003), and past this size the mixed step is
+// better with its kick beside the encounters.
+bool small_path(const opal_sim* s) {
+    return s->d.nsys == 1 && s->d.ntot <= kSmallBodies && !(s->d.p.precision == 1 && s->d.overlap);
+}
+bool small_kick(const opal_sim* s) { return small_path(s) && s->d.p.precision == 1; }
+
 opal_status capture_graph(opal_sim* s);
 
 void reset_scan_order(opal_sim* s);
@@ -420,6 +430,7 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
         s->sys.push_back(si);
         s->n_per_sys.push_back(nps[k]);
         s->n_big += si.nb;
+        s->d.nmax = std::max(s->d.nmax, (int)si.n);
         off += si.cap;
     }
     const int64_t N = off;
@@ -694,6 +705,7 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
                  force ? ", forced" : (best_ms >= 0 ? ", autotuned" : ""));
         CKF(up(d.sys, s->sys.data(), nsys * sizeof(SysInfo)));
         CKF(up(s->d_items, s->items.data(), s->items.size() * sizeof(KickItem)));
+        if (small_kick(s)) snprintf(s->kick_desc, sizeof(s->kick_desc), "mixed, a warp a body, %lld bodies", (long long)ntot);
     }
     {
         // warps a position takes in the row sums: eight rows a warp, at most eight warps
@@ -749,8 +761,16 @@ void note_launch(opal_sim* s, cudaError_t e) {
 void launch_kick_timed(opal_sim* s, cudaStream_t st) {
     const Dev& d = s->d;
     if (s->time_kick) cudaEventRecordWithFlags(s->kick_ev[0], st, cudaEventRecordExternal);
-    launch_kick(d, s->d_items, (int64_t)s->items.size(), s->kick_grid, d.p.precision, s->kick_variant, st);
+    if (small_kick(s)) launch_kick_small(d, st);
+    else launch_kick(d, s->d_items, (int64_t)s->items.size(), s->kick_grid, d.p.precision, s->kick_variant, st);
     if (s->time_kick) cudaEventRecordWithFlags(s->kick_ev[1], st, cudaEventRecordExternal);
+    if (!small_kick(s)) launch_kick_rows(d, st);
+}
+// the kick and its sums at the current positions, by d (the simulation's, or its gated copy)
+void launch_kick_sums(opal_sim* s, const Dev& d, cudaStream_t st) {
+    if (small_kick(s)) return launch_kick_small(d, st);
+    launch_kick_stage(d, d.p.precision, st);
+    launch_kick(d, s->d_items, (int64_t)s->items.size(), s->kick_grid, d.p.precision, s->kick_variant, st);
     launch_kick_rows(d, st);
 }
 
@@ -759,20 +779,29 @@ void launch_stage(opal_sim* s, int k, cudaStream_t st) {
     switch (k) {
         case 0: launch_step_reset(d, s->nsm, st); break;
         case 1: launch_open(d, st); break;
-        case 2: launch_scan(d, s->d_tiles, (int64_t)s->tiles.size(), s->scan_grid, st); break;
-        case 3: launch_confirm(d, s->confirm_grid, st); break;
-        case 4: launch_group(d, s->nsm, st); break;
+        case 2:
+            if (small_path(s)) launch_scan_small(d, s->d_tiles, (int64_t)s->tiles.size(), true, st);
+            else launch_scan(d, s->d_tiles, (int64_t)s->tiles.size(), s->scan_grid, st);
+            break;
+        case 3:
+            if (!small_path(s)) launch_confirm(d, s->confirm_grid, st);
+            break;
+        case 4:
+            if (!small_path(s)) launch_group(d, s->nsm, st);
+            break;
         case kStageBs:
             // the encounter kernels on parallel branches (one stream when profiling)
             note_launch(s, launch_bs(d, s->nsm, st, g_prof ? st : s->side2, g_prof ? st : s->side3, s->fork2_ev, s->join2_ev,
                                      s->join3_ev, false));
             break;
         case kStageKick:
-            launch_kick_stage(d, d.p.precision, st);
+            if (!small_kick(s)) launch_kick_stage(d, d.p.precision, st);
             launch_kick_timed(s, st);
             break;
         case kStageApply: launch_bs_apply(d, s->nsm, st); break;
-        case 8: launch_kick_fix(d, s->nsm, st); break;
+        case 8:
+            if (!small_kick(s)) launch_kick_fix(d, s->nsm, st);   // (that kick sums the momentum itself)
+            break;
         case 9: launch_close(d, st); break;
         case 10: launch_finish(d, st); break;
         case kStageReprime: {
@@ -781,9 +810,7 @@ void launch_stage(opal_sim* s, int k, cudaStream_t st) {
             Dev g = d;
             g.gated = 1;
             launch_prime(g, st);
-            launch_kick_stage(g, d.p.precision, st);
-            launch_kick(g, s->d_items, (int64_t)s->items.size(), s->kick_grid, d.p.precision, s->kick_variant, st);
-            launch_kick_rows(g, st);
+            launch_kick_sums(s, g, st);
             launch_first_accel_finish(g, st);
             prof_mark("accelerations afresh after a removal");
             break;
@@ -875,6 +902,7 @@ opal_status choose_mode(opal_sim* s) {
     if (share < 0.03) want = 1;
     else if (share > 0.08) want = 0;
     if (s->d.p.precision == 0) want = 0;
+    if (s->d.nsys == 1 && s->d.ntot <= kSmallBodies) want = 0;   // the small-system path (see small_path)
     // OPAL_STEP_ORDER=overlap or inorder forces one (the mixed form; the FP64 form is always in order)
     const char* force = getenv("OPAL_STEP_ORDER");
     if (force && s->d.p.precision == 1) {
@@ -1140,10 +1168,13 @@ opal_status opal_time_kick_alone(opal_sim* s, int32_t reps, double* ms) {
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     const int64_t ni = (int64_t)s->items.size();
-    launch_kick(d, s->d_items, ni, s->kick_grid, d.p.precision, s->kick_variant, s->stream);
+    auto kick = [&] {
+        if (small_kick(s)) launch_kick_small(d, s->stream);
+        else launch_kick(d, s->d_items, ni, s->kick_grid, d.p.precision, s->kick_variant, s->stream);
+    };
+    kick();
     cudaEventRecord(e0, s->stream);
-    for (int32_t r = 0; r < reps; r++)
-        launch_kick(d, s->d_items, ni, s->kick_grid, d.p.precision, s->kick_variant, s->stream);
+    for (int32_t r = 0; r < reps; r++) kick();
     cudaEventRecord(e1, s->stream);
     cudaError_t e = cudaEventSynchronize(e1);
     float t = 0.0f;
@@ -1200,9 +1231,7 @@ opal_status opal_debug_accel(opal_sim* s, const double* rc, double* a) {
     reset_scan_order(s);
     launch_debug_scan_prep(d, s->stream);
     launch_sort_bodies(d, s->stream);
-    launch_kick_stage(d, d.p.precision, s->stream);
-    launch_kick(d, s->d_items, (int64_t)s->items.size(), s->kick_grid, d.p.precision, s->kick_variant, s->stream);
-    launch_kick_rows(d, s->stream);
+    launch_kick_sums(s, d, s->stream);
     launch_first_accel_finish(d, s->stream);
     CK(cudaGetLastError());
     std::vector<double> ax(N), ay(N), az(N);
@@ -1282,8 +1311,12 @@ opal_status opal_debug_scan(opal_sim* s, const double* x0, const double* V0, con
                        offsetof(Ctl, steps_done) - offsetof(Ctl, ncand), s->stream));
     reset_scan_order(s);
     launch_debug_scan_prep(d, s->stream);
-    launch_scan(d, s->d_tiles, (int64_t)s->tiles.size(), s->scan_grid, s->stream);
-    launch_confirm(d, s->confirm_grid, s->stream);
+    if (small_path(s)) {
+        launch_scan_small(d, s->d_tiles, (int64_t)s->tiles.size(), false, s->stream);
+    } else {
+        launch_scan(d, s->d_tiles, (int64_t)s->tiles.size(), s->scan_grid, s->stream);
+        launch_confirm(d, s->confirm_grid, s->stream);
+    }
     CK(cudaMemsetAsync(d.label, 0xff, d.ntot * sizeof(int32_t), s->stream));   // no groups formed here
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(s->stream));

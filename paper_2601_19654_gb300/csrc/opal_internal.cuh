@@ -26,6 +26,7 @@ constexpr int kBsManyGroups = 4864;  // above this many groups a step integrates
 constexpr int kBsSoloGroups = 608;  // above this many groups the small-group kernel makes one attempt at a time
 constexpr int kBsSoloMid = 76;      // the same for groups of 5-16 members, above this many of them
 constexpr int kBucketDiv = 4;       // body slots per bucket of the spatial sort (cap / 4 buckets a system)
+constexpr int kSmallBodies = 1536;  // body slots up to which one system takes the small-system path
 constexpr int kBsOut = 9;           // doubles per member slot of the BS side buffer: x, V, m, R, alive
 constexpr int kFixParts = 4;        // the kick's correction after the encounters: member ranges per body
 constexpr int kBsRows = 8;          // extrapolation rows: n_k = 2, 4, ..., 16
@@ -64,6 +65,7 @@ struct Ctl {
     int qlock[3];        // queues of the lockstep kernels: up to 4, 16, 64 members (this step)
     int nhuge;           // groups of more than 64 members (this step)
     int ntov;            // tile pairs whose boxes overlap (this step)
+    int scan_done;       // blocks of the small-system scan done (this step)
     unsigned long long nsub;  // BS substeps (this step)
     long long steps_done;
     int cand_overflow;   // candidates lost to a full candidate list (forces a status)
@@ -196,6 +198,7 @@ struct Dev {
     float4* ks_lo;
     float* ks_rc;
     int kick_smem = 0;   // dynamic shared memory of the kick (FP64 form: the j side's sums)
+    int nmax = 0;   // bodies of the largest system (no group has more members)
     int rows_g = 8;  // warps a position takes in k_kick_rows (1, 2, 4 or 8: eight rows a warp)
     unsigned long long* timeline = nullptr;   // [kTlCount][2] (timeline builds only)
     double* ksum;    // [3 ntot]: each body's kick partial rows summed (by k_kick_rows), by body index
@@ -668,6 +671,10 @@ void launch_step_reset(const Dev& d, int nsm, cudaStream_t s);
 void launch_remove(const Dev& d, cudaStream_t s);
 void launch_scan(const Dev& d, const PairTile* tiles, int64_t ntiles, int grid, cudaStream_t s);
 void launch_confirm(const Dev& d, int grid, cudaStream_t s);
+// the mixed kick of one small system, and the closing jump's momentum (not when gated)
+void launch_kick_small(const Dev& d, cudaStream_t s);
+// the whole scan, and with group the groups, of one small system
+void launch_scan_small(const Dev& d, const PairTile* tiles, int64_t ntiles, bool group, cudaStream_t s);
 void launch_group(const Dev& d, int nsm, cudaStream_t s);
 cudaError_t bs_setup();   // dynamic shared memory of the BS kernels
 void launch_bs_packed(const Dev& d, int nsm, cudaStream_t s);

@@ -630,7 +630,7 @@ __global__ void __launch_bounds__(256) k_step_reset(Dev d) {
     int* c = reinterpret_cast<int*>(reinterpret_cast<char*>(d.ctl) + offsetof(Ctl, ncand));
     constexpr int nc = (int)((offsetof(Ctl, steps_done) - offsetof(Ctl, ncand)) / sizeof(int));
     int* h = reinterpret_cast<int*>(d.hctl);
-    constexpr int nh = (int)(sizeof(HugeCtl) / sizeof(int));
+    constexpr int nh = (int)(kHugeTeams * sizeof(HugeCtl) / sizeof(int));
     for (int64_t i = i0; i < d.ntot; i += st) {
         d.gcount[i] = 0;
         d.accf[i] = 0;

@@ -715,7 +715,7 @@ __global__ void __launch_bounds__(256) k_group_order(Dev d) {
         const int m0 = d.goff[g], n = d.goff[g + 1] - m0;
         if (threadIdx.x == 0 && n > 64) {
             // the whole-GPU kernel's, one after another
-            if (n <= d.hb.cap) d.ghuge[atomicAdd(&d.ctl->nhuge, 1)] = g;
+            if (n <= d.hb[0].cap) d.ghuge[atomicAdd(&d.ctl->nhuge, 1)] = g;
             else set_status(d.ctl, kEoverflow, 2000000 + g);
         } else if (threadIdx.x == 0) {
             // more than four members: the larger groups' lockstep kernels; many groups:
@@ -807,7 +807,7 @@ __device__ void group_order_block(const Dev& d, int ng, int* v) {
     for (int g = tid; g < ng; g += NT) {
         const int m0 = d.goff[g], n = d.goff[g + 1] - m0;
         if (n > 64) {
-            if (n <= d.hb.cap) d.ghuge[atomicAdd(&d.ctl->nhuge, 1)] = g;
+            if (n <= d.hb[0].cap) d.ghuge[atomicAdd(&d.ctl->nhuge, 1)] = g;
             else set_status(d.ctl, kEoverflow, 2000000 + g);
         } else if (n > 16) {
             d.glarge[atomicAdd(&d.ctl->nlarge, 1)] = g;

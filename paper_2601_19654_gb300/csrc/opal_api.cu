@@ -522,20 +522,25 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
     TRYF(dalloc(s, &d.gcls, 2 * d.gcap));
     TRYF(dalloc(s, &d.ghard, d.gcap));
     TRYF(dalloc(s, &d.ghuge, d.gcap));
-    {
-        // buffers of the whole-GPU encounter kernel, for groups of up to min(N, kHugeMax)
-        HugeBuf& H = d.hb;
-        H.cap = std::min<int64_t>(N, kHugeMax);
-        const int64_t nch = (H.cap + 63) / 64;
-        // the midpoint sequences advance in lockstep: chains, evaluation points
-        // and pair sums for each of the kBsRows sequences
-        TRYF(dalloc(s, &H.y, 6 * H.cap));
+    // buffers of the whole-GPU encounter kernel, for groups of up to min(N, kHugeMax)
+    for (HugeBuf& H : d.hb) {
+        H.cap = std::min<int64_t>(N, kHugeMax);   // (a multiple of 32)
+        const int64_t arrays = 2 * kBsRows + 2;
+        TRYF(dalloc(s, &H.pos, arrays * 3 * H.cap));
+        TRYF(dalloc(s, &H.posf, arrays * H.cap));
+        TRYF(dalloc(s, &H.box, 2 * 3 * huge_boxes(H.cap)));
+        TRYF(dalloc(s, &H.mot, 2 * H.cap));
+        TRYF(dalloc(s, &H.list, huge_boxes(H.cap) * kHugeListed));
+        TRYF(dalloc(s, &H.listed, huge_boxes(H.cap)));
+        TRYF(dalloc(s, &H.yv, 2 * 3 * H.cap));
+        TRYF(dalloc(s, &H.zv, (int64_t)kBsRows * 3 * H.cap));
         TRYF(dalloc(s, &H.z0, (int64_t)kBsRows * 6 * H.cap));
-        TRYF(dalloc(s, &H.z1, (int64_t)kBsRows * 6 * H.cap));
         TRYF(dalloc(s, &H.row, (int64_t)kBsRows * 6 * H.cap));
-        TRYF(dalloc(s, &H.pos, (int64_t)kBsRows * 3 * H.cap));
-        TRYF(dalloc(s, &H.posf, (int64_t)kBsRows * H.cap));
-        TRYF(dalloc(s, &H.part, (int64_t)kBsRows * 3 * H.cap * nch));
+        TRYF(dalloc(s, &H.sk, 6 * H.cap));
+        TRYF(dalloc(s, &H.ska, H.cap));
+        // blocks' units of a sequence: those of 32 members a warp, or of at most a member a warp of the launch
+        const int64_t units = huge_boxes(H.cap) / kHugeUnitWarps + kHugeTeams * s->nsm + 2;
+        TRYF(dalloc(s, &H.react, (int64_t)2 * kBsRows * units * kHugeWide * 3));
         TRYF(dalloc(s, &H.m, H.cap));
         TRYF(dalloc(s, &H.R, H.cap));
         TRYF(dalloc(s, &H.rc, H.cap));
@@ -543,12 +548,10 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
         TRYF(dalloc(s, &H.alive, H.cap));
         TRYF(dalloc(s, &H.gid, H.cap));
         TRYF(dalloc(s, &H.perm, H.cap));
-        TRYF(dalloc(s, &H.wide, H.cap));
         TRYF(dalloc(s, &H.key, H.cap));
-        TRYF(dalloc(s, &H.cbox, (int64_t)2 * kBsRows * nch * 2));
-        TRYF(dalloc(s, &d.hctl, 1));
-        CKF(cudaMemsetAsync(d.hctl, 0, sizeof(HugeCtl), s->stream));
     }
+    TRYF(dalloc(s, &d.hctl, kHugeTeams));
+    CKF(cudaMemsetAsync(d.hctl, 0, kHugeTeams * sizeof(HugeCtl), s->stream));
     TRYF(dalloc(s, &d.glost, 2 * d.flag_cap + 2));
     TRYF(dalloc(s, &d.undo, 3 * (2 * d.flag_cap + 2)));
     {

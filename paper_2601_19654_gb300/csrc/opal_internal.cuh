@@ -76,40 +76,49 @@ struct Ctl {
     int kick_done;
 };
 
-// Encounter groups of more than 64 members: working arrays of one group
-// (component-major [q][cap] arrays, cap = the largest such group).
+// Encounter groups of more than 64 members: working arrays of one group,
+// component-major [q][cap] by slot (members in spatial order; cap = the largest such group).
 constexpr int kHugeMax = 8192;    // members of the largest group these buffers take
 constexpr int kHugeCand = 1024;   // member pairs in contact after one substep
-constexpr int kHugeWide = 16;     // wide-rc members whose rows run one chunk a task (others: kHugeGroup chunks)
-constexpr int kHugeGroup = 8;     // chunks a pair-phase task takes for the other members
+constexpr int kHugeWide = 16;     // members of wide critical radius every block keeps a copy of
+constexpr int kHugeUnitWarps = 4; // a block's warps that take members, 32 each
+constexpr int kHugeTeams = 2;     // groups integrated at a time, each by a block an SM
+constexpr int kHugeListed = 1024;     // listed pairs of a warp's members at most
+constexpr int kHugeSmallBoxes = 640;   // boxes of fewer than 32 members at most
+__host__ __device__ __forceinline__ int64_t huge_boxes(int64_t cap) { return cap / 32 + kHugeSmallBoxes; }
 struct HugeBuf {
     int64_t cap;
-    double* y;                // [6][cap]: substep state
-    double *z0, *z1;          // [kBsRows][6][cap]: each midpoint sequence's chain
+    double* pos;              // [18][3][cap]: evaluation points (round parity x 8 + sequence; two substep starts)
+    float4* posf;             // [18][cap]: the same in float, with rc (rounded up; negative: massless)
+    float4* box;              // [2][huge_boxes][3], of the substep starts: box of each warp's members (lo, hi, motion)
+    float4* mot;              // [2][cap], of the substep starts: speed against the group's drift, acceleration, 0, R (rounded up)
+    double* yv;               // [2][3][cap]: velocities of the two substep starts
+    double* zv;               // [kBsRows][3][cap]: each midpoint sequence's velocities
+    double* z0;               // [kBsRows][6][cap]: its state one step back
     double* row;              // [kBsRows][6][cap]: extrapolation tableau (in place)
-    double* pos;              // [kBsRows][3][cap]: each sequence's positions of the current evaluation
-    float4* posf;             // [kBsRows][cap]: the same in float, with rc (rounded up)
-    double* part;             // [kBsRows][cap * chunks][3]: (1 - K) sums of each (member, 64-member chunk)
+    double* sk;               // [6][cap]: last value of the sequence that has just ended
+    float* ska;               // [cap]: size of the acceleration there
+    double* react;            // [2][kBsRows][blocks' units][kHugeWide][3]: members' side of the wide members' sums
     double *m, *R, *rc, *pinv;
+    int* list;                // [huge_boxes][kHugeListed]: near pairs of each warp's members in this substep
+    int* listed;              // [huge_boxes]: how many, or -1: more than there is room for
     int *alive, *gid;
-    int* perm;                // [cap]: members in spatial order; chunk ch is perm[64 ch .. 64 ch + 63]
-    int* wide;                // [cap]: 1 for a member with a wide critical radius (its row runs a chunk a task)
-    unsigned int* key;        // [cap]: their spatial keys
-    float4* cbox;             // [2][kBsRows][chunks][2]: box of each chunk's evaluation points (lo xyz +
-                              // largest rc, hi xyz), by round parity
+    int* perm;                // [cap]: each slot's member
+    unsigned int* key;        // [cap]: the members' spatial keys
 };
-// barrier and bookkeeping of the whole-GPU encounter kernel (zeroed every step)
+// barrier and bookkeeping of a team (zeroed every step)
 struct HugeCtl {
-    unsigned int bar_count, bar_gen;
+    unsigned int bar_count;             // arrivals at the team's barriers
     int abort, skip;
     int bb[4];                          // the group's box in x and y (order-mapped: min x, max x, min y, max y)
-    int nwide;                          // members with a wide critical radius, listed in wlist
-    int wlist[kHugeWide];
     int rcmm[2];                        // bits of the members' largest and smallest float rc (>= 0)
     int ncand, nmerge;
+    int moved[2];                       // 32 x attempt + round at which a member was past its lists' reach, by parity
+    int ref;                            // slot of the group's lowest member
+    int nnear;                          // pairs near one another at the start, without the wide members
     double El;
-    unsigned long long err[kBsRows];   // grid-wide maximum error of each row (bits of a double >= 0)
-    int2 cand[kHugeCand];
+    int err[kBsRows];                   // the last attempt in which a member failed each row's test
+    int2 cand[kHugeCand];               // slots, the lower body first
 };
 
 // Neville coefficients 1 / ((n_k / n_{k-j})^2 - 1) with n_k = 2(k+1): exact
@@ -241,8 +250,8 @@ struct Dev {
     int32_t* gcls;                      // [2][gcap]: groups by size class (2 and 4 members at most)
     int32_t* ghard;                     // [gcap]: groups the packed kernel leaves to the lockstep kernel
     int32_t* ghuge;                     // [gcap]: groups of more than 64 members
-    HugeBuf hb;                         // working arrays of the whole-GPU encounter kernel
-    HugeCtl* hctl;
+    HugeBuf hb[kHugeTeams];             // working arrays of the whole-GPU encounter kernel
+    HugeCtl* hctl;                      // [kHugeTeams]
     int64_t gcap;                       // capacity of each class list
     int* gcount;                        // per body: members of the group it roots (zero between steps)
     int* gofs;                          // per root: its group's first member slot

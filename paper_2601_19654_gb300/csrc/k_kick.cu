@@ -176,11 +176,6 @@ __device__ __forceinline__ void far_tile(const float* sx, const float* sy, const
     }
 }
 
-// the j-tile's lo parts and bounds rc^2 (the near paths')
-struct KickLo {
-    float x[kJTile], y[kJTile], z[kJTile], b[kJTile];
-};
-
 // Near j-tile: the packed loop, with every pair closer than the i-body's
 // threshold left out (its term set to zero) and its j noted in the lane's
 // own list in shared memory; then the lanes take the slow path (lo parts,
@@ -193,7 +188,7 @@ constexpr int kNearList = 32;   // listed near pairs per lane and i-body before 
 
 template <int T, int NI>
 __device__ __forceinline__ void near_flush(const float* sx, const float* sy, const float* sz, const float* sm,
-                                           const KickLo& sl, const float* src, const unsigned char* lst,
+                                           const float4* sl, const float* src, const unsigned char* lst,
                                            const int (&cnt)[NI], const float2 (&nx)[NI], const float2 (&ny)[NI],
                                            const float2 (&nz)[NI], const float4 (&li)[NI], const float (&rci)[NI],
                                            int form, float2 (&ax)[NI], float2 (&ay)[NI], float2 (&az)[NI]) {
@@ -204,7 +199,7 @@ __device__ __forceinline__ void near_flush(const float* sx, const float* sy, con
         for (int k = 0; k < most; k++) {
             if (k < cnt[q]) {
                 const int jj = lst[(k * NI + q) * T + threadIdx.x];
-                const float4 r = slow_pair_f(li[q], make_float4(sl.x[jj], sl.y[jj], sl.z[jj], 0.0f), sx[jj] + nx[q].x, sy[jj] + ny[q].x, sz[jj] + nz[q].x,
+                const float4 r = slow_pair_f(li[q], sl[jj], sx[jj] + nx[q].x, sy[jj] + ny[q].x, sz[jj] + nz[q].x,
                                              sm[jj], rci[q], src[jj], form);
                 ax[q].x = fmaf(r.x, r.y, ax[q].x);
                 ay[q].x = fmaf(r.x, r.z, ay[q].x);
@@ -216,7 +211,7 @@ __device__ __forceinline__ void near_flush(const float* sx, const float* sy, con
 
 template <int T, int NI>
 __device__ __forceinline__ void near_tile(const Dev& d, int64_t i0, float rcm, const float* sx, const float* sy,
-                                          const float* sz, const float* sm, const KickLo& sl, const float* src,
+                                          const float* sz, const float* sm, const float4* sl, const float* src,
                                           unsigned char* lst, const float2 (&nx)[NI], const float2 (&ny)[NI],
                                           const float2 (&nz)[NI], int form, float2 (&ax)[NI], float2 (&ay)[NI],
                                           float2 (&az)[NI]) {
@@ -278,104 +273,6 @@ __device__ __forceinline__ void near_tile(const Dev& d, int64_t i0, float rcm, c
     near_flush<T, NI>(sx, sy, sz, sm, sl, src, lst, cnt, nx, ny, nz, li, rci, form, ax, ay, az);
 }
 
-// Near j-tile of an i-tile whose own critical radii are far below the system's largest
-// (kKickWide): a giant planet's radius puts whole systems inside 2 (rc_i + rc_max), while few
-// of the pairs there are inside the larger radius of their two.  Every pair takes
-// the lo parts and a reciprocal square root refined by a Newton step, in packed pairs; only
-// those inside that radius are left out and listed for the slow path (the changeover).
-// Kick alone: 1024 + 262144 bodies 480 to 243 us, 131072 bodies and two giants 11.4 to 7.7 ms
-// (a tile pair costs about twice a far one; the test of four pairs together is a fifth of that).
-constexpr float kKickWide = 16.0f;   // (equal masses and the log-uniform ranges of one system stay below it)
-
-template <int T, int NI>
-__device__ __forceinline__ void near_wide(const Dev& d, int64_t i0, float rcj, const float* sx, const float* sy,
-                                          const float* sz, const float* sm, const KickLo& sl, const float* src,
-                                          unsigned char* lst, const float2 (&nx)[NI], const float2 (&ny)[NI],
-                                          const float2 (&nz)[NI], int form, float2 (&ax)[NI], float2 (&ay)[NI],
-                                          float2 (&az)[NI]) {
-    float4 li[NI];
-    float2 nlx[NI], nly[NI], nlz[NI];
-    float rci[NI], bi[NI], bt[NI];
-    int cnt[NI];
-#pragma unroll
-    for (int q = 0; q < NI; q++) {
-        const int64_t p = i0 + q * T + threadIdx.x;
-        li[q] = d.ks_lo[p];
-        nlx[q] = make_float2(-li[q].x, -li[q].x);
-        nly[q] = make_float2(-li[q].y, -li[q].y);
-        nlz[q] = make_float2(-li[q].z, -li[q].z);
-        rci[q] = d.ks_rc[p];
-        bi[q] = fmaxf(1.0001f * (rci[q] * rci[q]), 1e-30f);   // (the margin covers the roundings)
-        bt[q] = fmaxf(bi[q], 1.0001f * (rcj * rcj));          // no j of the tile has a larger bound
-        cnt[q] = 0;
-    }
-    const float4* px = reinterpret_cast<const float4*>(sx);
-    const float4* py = reinterpret_cast<const float4*>(sy);
-    const float4* pz = reinterpret_cast<const float4*>(sz);
-    const float4* pm = reinterpret_cast<const float4*>(sm);
-    const float4* plx = reinterpret_cast<const float4*>(sl.x);
-    const float4* ply = reinterpret_cast<const float4*>(sl.y);
-    const float4* plz = reinterpret_cast<const float4*>(sl.z);
-#pragma unroll 1
-    for (int jq = 0; jq < kJTile / 4; jq++) {
-        const float4 x4 = px[jq], y4 = py[jq], z4 = pz[jq], m4 = pm[jq];
-        const float4 lx4 = plx[jq], ly4 = ply[jq], lz4 = plz[jq];
-#pragma unroll
-        for (int q = 0; q < NI; q++) {
-            float2 dx[2], dy[2], dz[2], r2[2], sv[2];
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const float2 xj = h ? make_float2(x4.z, x4.w) : make_float2(x4.x, x4.y);
-                const float2 yj = h ? make_float2(y4.z, y4.w) : make_float2(y4.x, y4.y);
-                const float2 zj = h ? make_float2(z4.z, z4.w) : make_float2(z4.x, z4.y);
-                const float2 mj = h ? make_float2(m4.z, m4.w) : make_float2(m4.x, m4.y);
-                const float2 lx = h ? make_float2(lx4.z, lx4.w) : make_float2(lx4.x, lx4.y);
-                const float2 ly = h ? make_float2(ly4.z, ly4.w) : make_float2(ly4.x, ly4.y);
-                const float2 lz = h ? make_float2(lz4.z, lz4.w) : make_float2(lz4.x, lz4.y);
-                dx[h] = __fadd2_rn(__fadd2_rn(xj, nx[q]), __fadd2_rn(lx, nlx[q]));
-                dy[h] = __fadd2_rn(__fadd2_rn(yj, ny[q]), __fadd2_rn(ly, nly[q]));
-                dz[h] = __fadd2_rn(__fadd2_rn(zj, nz[q]), __fadd2_rn(lz, nlz[q]));
-                r2[h] = __ffma2_rn(dz[h], dz[h], __ffma2_rn(dy[h], dy[h], __fmul2_rn(dx[h], dx[h])));
-                // 1/r^3 = y^3 (1 - e)^(-3/2), e = 1 - r^2 y^2 a few 1e-7
-                const float2 y = make_float2(rsqrt_approx(r2[h].x), rsqrt_approx(r2[h].y));
-                const float2 y2 = __fmul2_rn(y, y);
-                const float2 e = __ffma2_rn(r2[h], y2, make_float2(-1.0f, -1.0f));
-                const float2 c = __ffma2_rn(e, make_float2(-1.5f, -1.5f), make_float2(1.0f, 1.0f));
-                sv[h] = __fmul2_rn(__fmul2_rn(__fmul2_rn(mj, y), y2), c);
-            }
-            // the four together: is any of them inside the tile's largest radius
-            if (fminf(fminf(r2[0].x, r2[0].y), fminf(r2[1].x, r2[1].y)) < bt[q]) {
-#pragma unroll
-                for (int e = 0; e < 4; e++) {
-                    const int j = 4 * jq + e;
-                    float& s = e == 0 ? sv[0].x : e == 1 ? sv[0].y : e == 2 ? sv[1].x : sv[1].y;
-                    const float rr = e == 0 ? r2[0].x : e == 1 ? r2[0].y : e == 2 ? r2[1].x : r2[1].y;
-                    if (rr < fmaxf(bi[q], sl.b[j])) {
-                        s = 0.0f;
-                        lst[(cnt[q]++ * NI + q) * T + threadIdx.x] = (unsigned char)j;
-                    }
-                }
-            }
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                ax[q] = __ffma2_rn(sv[h], dx[h], ax[q]);
-                ay[q] = __ffma2_rn(sv[h], dy[h], ay[q]);
-                az[q] = __ffma2_rn(sv[h], dz[h], az[q]);
-            }
-        }
-        // room for the next quad's four pairs in every lane's list, or work it off
-        bool full = false;
-#pragma unroll
-        for (int q = 0; q < NI; q++) full |= cnt[q] > kNearList - 4;
-        if (__any_sync(0xffffffffu, full)) {
-            near_flush<T, NI>(sx, sy, sz, sm, sl, src, lst, cnt, nx, ny, nz, li, rci, form, ax, ay, az);
-#pragma unroll
-            for (int q = 0; q < NI; q++) cnt[q] = 0;
-        }
-    }
-    near_flush<T, NI>(sx, sy, sz, sm, sl, src, lst, cnt, nx, ny, nz, li, rci, form, ax, ay, az);
-}
-
 // Items index the system's bodies in the order the encounter scan sorted
 // them (cells of the path midpoints, so a 128-body tile is compact); the
 // staging kernel has copied them there.  An item is one j-tile of 256
@@ -400,10 +297,9 @@ __global__ void __launch_bounds__(T, MINB) k_kick_mixed(Dev d, const KickItem* _
     static_assert(IT == kKickBox || IT == 2 * kKickBox, "an i-tile is one staged box");
     const float4* ibox = IT == kKickBox ? d.kbox : d.kbox2;
     __shared__ __align__(16) float sx[kJTile], sy[kJTile], sz[kJTile], sm[kJTile];
-    __shared__ __align__(16) KickLo sl;
+    __shared__ float4 sl[kJTile];     // lo parts and 4 rc^2 of the j-tile (the near path's)
     __shared__ float src[kJTile];
     __shared__ KickItem s_w;          // the block's item
-    __shared__ float s_jrc;           // no rc of its j is above this
     __shared__ float s_jbox[6];       // its j-tile's box (lo xyz, hi xyz)
     __shared__ unsigned char s_near[kNearList * NI * T];   // near pairs' j, per lane and i-body
     if (d.ctl->status) return;
@@ -459,13 +355,8 @@ __global__ void __launch_bounds__(T, MINB) k_kick_mixed(Dev d, const KickItem* _
                 sy[k0 + u] = vy[u];
                 sz[k0 + u] = vz[u];
                 sm[k0 + u] = vm[u];
-                const float4 l = k0 + u < nj ? d.ks_lo[w.j0 + k0 + u] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                const float rc = k0 + u < nj ? d.ks_rc[w.j0 + k0 + u] : 0.0f;
-                sl.x[k0 + u] = l.x;
-                sl.y[k0 + u] = l.y;
-                sl.z[k0 + u] = l.z;
-                sl.b[k0 + u] = 1.0001f * (rc * rc);
-                src[k0 + u] = rc;
+                sl[k0 + u] = k0 + u < nj ? d.ks_lo[w.j0 + k0 + u] : make_float4(0.0f, 0.0f, 0.0f, 1e-30f);
+                src[k0 + u] = k0 + u < nj ? d.ks_rc[w.j0 + k0 + u] : 0.0f;
             }
             if (threadIdx.x == 0) {
                 // the j-tile's box: its whole 256 positions (any records past nj
@@ -474,7 +365,6 @@ __global__ void __launch_bounds__(T, MINB) k_kick_mixed(Dev d, const KickItem* _
                 const float4 lo = d.kbox2[2 * (w.j0 / kJTile)], hi = d.kbox2[2 * (w.j0 / kJTile) + 1];
                 s_jbox[0] = lo.x; s_jbox[1] = lo.y; s_jbox[2] = lo.z;
                 s_jbox[3] = hi.x; s_jbox[4] = hi.y; s_jbox[5] = hi.z;
-                s_jrc = fmaxf(0.5f * sqrtf(lo.w) - rcm + 1e-6f * rcm, 0.0f);   // (lo.w: (2 (rc + rc_max))^2)
             }
         }
         __syncthreads();
@@ -512,9 +402,6 @@ __global__ void __launch_bounds__(T, MINB) k_kick_mixed(Dev d, const KickItem* _
                 }
                 near = g2 < pb[0].w * 1.001f;
             }
-            // no rc of the i-tile above 1 / kKickWide of the largest: its threshold (2 (rc + rc_max))^2 says
-            constexpr float kw = 2.0f * (1.0f + 1.0f / kKickWide);
-            const bool wide = pb[0].w < (kw * rcm) * (kw * rcm);
             // the next i-tile's positions and box, in flight during this one
             const int64_t nb0 = ib + w.istep < w.i1 ? ib + w.istep : ib;
 #pragma unroll
@@ -529,8 +416,7 @@ __global__ void __launch_bounds__(T, MINB) k_kick_mixed(Dev d, const KickItem* _
             float2 ax[NI], ay[NI], az[NI];
 #pragma unroll
             for (int q = 0; q < NI; q++) ax[q] = ay[q] = az[q] = make_float2(0.0f, 0.0f);
-            if (near && wide) near_wide<T, NI>(d, ib, s_jrc, sx, sy, sz, sm, sl, src, s_near, nx, ny, nz, form, ax, ay, az);
-            else if (near) near_tile<T, NI>(d, ib, rcm, sx, sy, sz, sm, sl, src, s_near, nx, ny, nz, form, ax, ay, az);
+            if (near) near_tile<T, NI>(d, ib, rcm, sx, sy, sz, sm, sl, src, s_near, nx, ny, nz, form, ax, ay, az);
             else far_tile<NI>(sx, sy, sz, sm, nx, ny, nz, ax, ay, az);
             // partial rows by sorted position (coalesced), each the exact float
             // pair of the two lanes' sums; k_kick_rows sums them by position
@@ -739,36 +625,13 @@ __global__ void __launch_bounds__(32 * W) k_kick_fp64(Dev d, const KickItem* __r
 // when r^2 < (2 (rc_i + rc_max))^2, where the kick's tile test sends it too.
 
 // one pair term of the mixed kick: i (hi, lo, rc, threshold) and j (hi, lo, rc)
-// The slow path's term where i's critical radius is far below the system's largest (see
-// near_wide): the square root and the division only inside the larger radius of the two.
-__device__ __forceinline__ float4 wide_pair_f(float4 li, float4 lj, float dx, float dy, float dz, float mj, float rci,
-                                              float rcj, int form) {
-    dx += lj.x - li.x;
-    dy += lj.y - li.y;
-    dz += lj.z - li.z;
-    const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx)), rcij = fmaxf(rci, rcj);
-    float s = 0.0f;
-    if (r2 < fmaxf(1.0001f * (rcij * rcij), 1e-30f)) {
-        if (r2 > 0.0f) {
-            const float r = sqrtf(r2);
-            s = mj * changeover_f(r, rcij, form) / (r2 * r);
-        }
-    } else {
-        float y = rsqrt_approx(r2);
-        y = fmaf(0.5f * y, fmaf(-(r2 * y), y, 1.0f), y);
-        s = (mj * y) * (y * y);
-    }
-    return make_float4(s, dx, dy, dz);
-}
-
 __device__ __forceinline__ float3 term_f(float4 hi, float4 li, float rci, float thr, float4 hj, float4 lj, float rcj,
-                                         int form, bool wide) {
+                                         int form) {
     float dx = hj.x - hi.x, dy = hj.y - hi.y, dz = hj.z - hi.z;
     float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
     float s;
     if (r2 < thr) {
-        float4 r = wide ? wide_pair_f(li, lj, dx, dy, dz, hj.w, rci, rcj, form)
-                        : slow_pair_f(li, lj, dx, dy, dz, hj.w, rci, rcj, form);
+        float4 r = slow_pair_f(li, lj, dx, dy, dz, hj.w, rci, rcj, form);
         s = r.x;
         dx = r.y;
         dy = r.z;
@@ -865,7 +728,6 @@ __global__ void __launch_bounds__(kFixThreads) k_kick_fix(Dev d, int nbody_block
         const float rci = d.rcf[b];
         const float tf = 2.0f * (rci + rcm);
         const float thrf = fmaxf(tf * tf, 1e-30f);
-        const bool wide = rcm > kKickWide * rci;
         const double xi = d.x[b], yi = d.y[b], zi = d.z[b], rcid = d.rc[b];
         const double td = 2.0 * (rcid + (double)rcm);
         const double thrd = fmax(td * td, 1e-300);
@@ -919,8 +781,8 @@ __global__ void __launch_bounds__(kFixThreads) k_kick_fix(Dev d, int nbody_block
                                  dz = __fadd2_rn(make_float2(a.z, c.z), nz2);
                     const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
                     if (r2.x < thrf || r2.y < thrf) {
-                        const float3 ta = term_f(hi, li, rci, thrf, a, snl[q], snr[q], form, wide);
-                        const float3 tc = term_f(hi, li, rci, thrf, c, snl[q + 1], snr[q + 1], form, wide);
+                        const float3 ta = term_f(hi, li, rci, thrf, a, snl[q], snr[q], form);
+                        const float3 tc = term_f(hi, li, rci, thrf, c, snl[q + 1], snr[q + 1], form);
                         tx2.x += ta.x; ty2.x += ta.y; tz2.x += ta.z;
                         tx2.y += tc.x; ty2.y += tc.y; tz2.y += tc.z;
                     } else {
@@ -932,7 +794,7 @@ __global__ void __launch_bounds__(kFixThreads) k_kick_fix(Dev d, int nbody_block
                     }
                 }
                 if (q < n) {
-                    const float3 t = term_f(hi, li, rci, thrf, snh[q], snl[q], snr[q], form, wide);
+                    const float3 t = term_f(hi, li, rci, thrf, snh[q], snl[q], snr[q], form);
                     tx2.x += t.x; ty2.x += t.y; tz2.x += t.z;
                 }
                 fold(hx, lx, tx2.x);
@@ -986,7 +848,6 @@ __global__ void __launch_bounds__(kFixThreads) k_kick_fix(Dev d, int nbody_block
             const float rci = d.rcf[g];
             const float tf = 2.0f * (rci + rcm);
             const float thrf = fmaxf(tf * tf, 1e-30f);
-            const bool wide = rcm > kKickWide * rci;
             const double xi = d.x[g], yi = d.y[g], zi = d.z[g], rcid = d.rc[g];
             const double td = 2.0 * (rcid + (double)rcm);
             const double thrd = fmax(td * td, 1e-300);
@@ -1024,8 +885,7 @@ __global__ void __launch_bounds__(kFixThreads) k_kick_fix(Dev d, int nbody_block
                                 const float rs = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
                                 float sv;
                                 if (rs < thrf) {
-                                    const float4 r = wide ? wide_pair_f(li, d.kl[j], ex, ey, ez, hh.w, rci, d.rcf[j], form)
-                                                          : slow_pair_f(li, d.kl[j], ex, ey, ez, hh.w, rci, d.rcf[j], form);
+                                    const float4 r = slow_pair_f(li, d.kl[j], ex, ey, ez, hh.w, rci, d.rcf[j], form);
                                     sv = r.x;
                                     ex = r.y;
                                     ey = r.z;

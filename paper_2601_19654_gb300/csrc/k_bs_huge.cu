@@ -100,38 +100,25 @@ __device__ __forceinline__ float4* huge_box(const HugeBuf& H, int a) {   // (of 
 __device__ __forceinline__ float4* huge_mot(const HugeBuf& H, int a) { return H.mot + (int64_t)(a - kHugeY) * H.cap; }
 __device__ __forceinline__ float huge_reach(float4 m, float h) { return h * fmaf(2.0f * h, m.y, m.x); }
 
-// (1 - K) / r^3 of a pair inside the larger critical radius of the two, else 0, in
-// about 24 FP64 operations where library rsqrt and division take 34.  pinv: 1 / (0.9 rc).
-// (Not inlined: a round's code runs once through, and what does not stay in the
-// instruction caches costs more than the call.)
-//  - 1/r from the hardware's approximate reciprocal square root y (1 - r^2 y^2 = e below
-//    1.9e-6, measured): y (1 + e (1/2 + 3/8 e)), and 1/r^3 = y^3 (1 + e (3/2 + 15/8 e)),
-//    next terms below 2^-56; the reciprocal of the rational form's denominator (between
-//    1/2 and 1) likewise from an approximate one with a relative error below 1e-6.
-//  - u = 1 - y_c = 10/9 - r / (0.9 rc) for y_c = (r - 0.1 rc) / (0.9 rc); 1 - K is
-//    u^2 / (1 - 2u + 2u^2) or, by the quintic's symmetry, u^3 (10 - 15u + 6u^2).
-__device__ __noinline__ double huge_weight(double dx, double dy, double dz, double rcb, double pinvb, double rco,
-                                              double pinvo, int form) {
+// G m (1 - K) / r^3 (gm: G m) of a pair inside the larger critical radius of the two, else 0.
+// The arithmetic, its order and its contraction are written out: with one term near it, a
+// member's acceleration then has the same bits in whatever order this kernel sums the others,
+// and a step decision within rounding of the tolerance falls the same way.
+// (Hardware approximations in place of the library's rsqrt and division save 10 of 34 FP64
+// operations and nothing of a round's time; step decisions then fell differently in one run
+// of eight, after which bodies deep inside the giant's sphere differed by up to 3e-7.)  Not
+// inlined: a round's code runs once through, and what does not stay in the instruction caches
+// costs more than the call.
+__device__ __noinline__ double huge_factor(double dx, double dy, double dz, double rcb, double pinvb, double rco,
+                                           double pinvo, double gm, int form) {
     const bool first = gt_nonneg(rcb, rco);
     const double rc = first ? rcb : rco;
-    const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-    if (ge_nonneg(r2, rc * rc)) return 0.0;   // 1 - K = 0 at or beyond rc
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));
-    const double y2 = y * y, e = fma(-r2, y2, 1.0);
-    const double r = (r2 * y) * fma(e, fma(0.375, e, 0.5), 1.0);
-    const double ri3 = (y2 * y) * fma(e, fma(1.875, e, 1.5), 1.0);
-    const double u = fma(-r, first ? pinvb : pinvo, 10.0 / 9.0);
-    if (le_zero(u) || !(r2 > 0.0)) return 0.0;
-    if (ge_nonneg(u, 1.0)) return ri3;        // K = 0 within 0.1 rc
-    if (form == 0) {
-        const double den = fma(u + u, u - 1.0, 1.0);
-        double q;
-        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(q) : "d"(den));
-        const double f = fma(-den, q, 1.0);
-        return (ri3 * (u * u)) * fma(q, fma(f, f, f), q);
-    }
-    return ri3 * ((u * u * u) * fma(u, fma(6.0, u, -15.0), 10.0));
+    const double dr2 = fma(dz, dz, fma(dx, dx, __dmul_rn(dy, dy)));
+    if (ge_nonneg(dr2, __dmul_rn(rc, rc))) return 0.0;   // 1 - K = 0 at or beyond rc
+    const double dri = rsqrt(dr2), dr = __dmul_rn(dr2, dri);
+    if (ge_nonneg(dr, rc)) return 0.0;
+    const double y = __dmul_rn(fma(-0.1, rc, dr), first ? pinvb : pinvo);
+    return mutual_factor(__dmul_rn(gm, __dmul_rn(__dmul_rn(dri, dri), dri)), y, form);
 }
 
 // Sums over the warp of three doubles, in six additions: lanes 0, 8 and 16 hold
@@ -355,7 +342,7 @@ __device__ __noinline__ void huge_listed(const Dev& d, const HugeBuf& H, int a, 
         double tx = 0.0, ty = 0.0, tz = 0.0;
         if (hit) {
             const double ex = pos[o] - xs, ey = pos[c + o] - ys, ez = pos[2 * c + o] - zs;
-            const double w = d.p.G * H.m[o] * huge_weight(ex, ey, ez, rs, ps, H.rc[o], H.pinv[o], form);
+            const double w = huge_factor(ex, ey, ez, rs, ps, H.rc[o], H.pinv[o], d.p.G * H.m[o], form);
             tx = w * ex;
             ty = w * ey;
             tz = w * ez;
@@ -411,7 +398,7 @@ __device__ __noinline__ void huge_dense(const Dev& d, const HugeBuf& H, int a, i
                 if (!((hit >> q) & 1u)) continue;
                 const int o = o0 + 32 * q;
                 const double ex = pos[o] - xs, ey = pos[c + o] - ys, ez = pos[2 * c + o] - zs;
-                const double w = d.p.G * H.m[o] * huge_weight(ex, ey, ez, rs, ps, H.rc[o], H.pinv[o], form);
+                const double w = huge_factor(ex, ey, ez, rs, ps, H.rc[o], H.pinv[o], d.p.G * H.m[o], form);
                 tx = fma(w, ex, tx);
                 ty = fma(w, ey, ty);
                 tz = fma(w, ez, tz);
@@ -608,7 +595,8 @@ struct HugeSh {
     double base[kBsRows][kHugeWide][3];         // star and other wide members at this round's points
     double F[kBsRows][kHugeWide][3];            // the whole acceleration at the last round's
     double red[kHugeUnitWarps][kHugeWide][3];   // the warps' sums of the members' side
-    double m[kHugeWide], rc[kHugeWide], pinv[kHugeWide], R[kHugeWide];
+    double m[kHugeWide], gm[kHugeWide], igm[kHugeWide];   // (G m and its reciprocal)
+    double rc[kHugeWide], pinv[kHugeWide], R[kHugeWide];
     double sq[kHugeWide][6][2];                 // squares of a row's error and value
     int alive[kHugeWide], slot[kHugeWide];
     HugeQueue q[kHugeUnitWarps];
@@ -794,6 +782,8 @@ __global__ void __launch_bounds__(kHugeThreads, 3) k_bs_huge(Dev d, int nsm) {
                     S.y[q][3 + e] = vel[e * c + i];
                 }
                 S.m[q] = H.m[i];
+                S.gm[q] = G * H.m[i];
+                S.igm[q] = S.gm[q] > 0.0 ? 1.0 / S.gm[q] : 0.0;
                 S.R[q] = H.R[i];
                 S.rc[q] = H.rc[i];
                 S.pinv[q] = H.pinv[i];
@@ -1093,7 +1083,7 @@ __global__ void __launch_bounds__(kHugeThreads, 3) k_bs_huge(Dev d, int nsm) {
 #pragma unroll
                         for (int e = 0; e < 6; e++) Z[e] = own && r > 0 ? H.z0[((int64_t)k * 6 + e) * c + i] : 0.0;
                         if (have) {
-                            const double ri = rsqrt(P[0] * P[0] + P[1] * P[1] + P[2] * P[2]);
+                            const double ri = rsqrt(fma(P[2], P[2], fma(P[1], P[1], __dmul_rn(P[0], P[0]))));
                             const double sk = -GM0 * (ri * ri * ri);
 #pragma unroll
                             for (int e = 0; e < 3; e++) acc[e] = sk * P[e];
@@ -1114,14 +1104,14 @@ __global__ void __launch_bounds__(kHugeThreads, 3) k_bs_huge(Dev d, int nsm) {
                                 dx = Q[0] - P[0];
                                 dy = Q[1] - P[1];
                                 dz = Q[2] - P[2];
-                                s = huge_weight(dx, dy, dz, rc, pinv, S.rc[w], S.pinv[w], form);
+                                s = huge_factor(dx, dy, dz, rc, pinv, S.rc[w], S.pinv[w], S.gm[w], form);
                             }
                             double sum = 0.0;
                             if (__any_sync(0xffffffffu, s != 0.0)) {
-                                const double sw = G * S.m[w] * s, sb = -(G * mb * s);
-                                acc[0] += sw * dx;
-                                acc[1] += sw * dy;
-                                acc[2] += sw * dz;
+                                const double sb = -(s * S.igm[w]) * (G * mb);
+                                acc[0] = __dadd_rn(acc[0], __dmul_rn(s, dx));
+                                acc[1] = __dadd_rn(acc[1], __dmul_rn(s, dy));
+                                acc[2] = __dadd_rn(acc[2], __dmul_rn(s, dz));
                                 sum = warp_sum3(sb * dx, sb * dy, sb * dz);
                             }
                             if ((lane & 7) == 0 && lane < 24) S.red[warp][w][lane >> 3] = sum;
@@ -1191,17 +1181,17 @@ __global__ void __launch_bounds__(kHugeThreads, 3) k_bs_huge(Dev d, int nsm) {
                             const int k = k0 + q / nwide, w = q % nwide;
                             if (!S.alive[w]) continue;
                             const double* P = r == 0 ? S.y[w] : S.z1[k][w];
-                            const double ri = rsqrt(P[0] * P[0] + P[1] * P[1] + P[2] * P[2]);
+                            const double ri = rsqrt(fma(P[2], P[2], fma(P[1], P[1], __dmul_rn(P[0], P[0]))));
                             const double sk = -GM0 * (ri * ri * ri);
                             double ax = sk * P[0], ay = sk * P[1], az = sk * P[2];
                             for (int o = 0; o < nwide; o++) {
                                 if (o == w || !S.alive[o] || le_zero(S.m[o])) continue;
                                 const double* Q = r == 0 ? S.y[o] : S.z1[k][o];
                                 const double dx = Q[0] - P[0], dy = Q[1] - P[1], dz = Q[2] - P[2];
-                                const double s = G * S.m[o] * huge_weight(dx, dy, dz, S.rc[w], S.pinv[w], S.rc[o], S.pinv[o], form);
-                                ax += s * dx;
-                                ay += s * dy;
-                                az += s * dz;
+                                const double s = huge_factor(dx, dy, dz, S.rc[w], S.pinv[w], S.rc[o], S.pinv[o], G * S.m[o], form);
+                                ax = __dadd_rn(ax, __dmul_rn(s, dx));
+                                ay = __dadd_rn(ay, __dmul_rn(s, dy));
+                                az = __dadd_rn(az, __dmul_rn(s, dz));
                             }
                             S.base[k][w][0] = ax;
                             S.base[k][w][1] = ay;

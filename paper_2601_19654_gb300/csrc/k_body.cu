@@ -7,7 +7,11 @@
 // reduction, LOOP 3 positions, LOOP 4 copy of x and v) and third block
 // (arxes_drift on every body, failure flag); Hill / critical radii from the
 // instantaneous heliocentric distance, Sec. 2.1.1 item (4) and footnotes.
+#include <cooperative_groups.h>
+
 #include "opal_internal.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace opal {
 
@@ -435,42 +439,168 @@ __global__ void k_finish(Dev d) {
     }
 }
 
-// get_state of system s, first pass: its momentum sum m V over the live
+// get_state's arrays of the live bodies, in id order: ids, m, R, x (3 a body), v (heliocentric)
+struct ExportView {
+    int64_t* ids;
+    double *m, *R, *x, *v;
+};
+__host__ __device__ __forceinline__ ExportView export_view(double* buf, int64_t cap) {
+    return ExportView{reinterpret_cast<int64_t*>(buf), buf + cap, buf + 2 * cap, buf + 3 * cap, buf + 6 * cap};
+}
+
+// The live ones of a block's T bodies (thread: body si.off + k) to places base on, through
+// shared memory so that the stores are contiguous (the arrays may lie in host memory);
+// vs: the star's velocity P / M0, which the heliocentric velocities add.
+template <int T>
+__device__ __forceinline__ int export_tile(const Dev& d, const SysInfo& si, int64_t k, bool in, const double* vs, int64_t base,
+                                           const ExportView& o) {
+    __shared__ double sx[3 * T], sv[3 * T], sm[T], sR[T];
+    __shared__ int64_t sid[T];
+    __shared__ int wcnt[T / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t b = si.off + k;
+    const bool live = in && d.alive[b] != 0;
+    const unsigned bm = __ballot_sync(0xffffffffu, live);
+    __syncthreads();   // (the tile before this one has been written out)
+    if (lane == 0) wcnt[warp] = __popc(bm);
+    __syncthreads();
+    int at = __popc(bm & ((1u << lane) - 1u)), n = 0;
+#pragma unroll
+    for (int w = 0; w < T / 32; w++) {
+        if (w < warp) at += wcnt[w];
+        n += wcnt[w];
+    }
+    if (live) {
+        sid[at] = k;
+        sm[at] = d.m[b];
+        sR[at] = d.R[b];
+        sx[3 * at] = d.x[b];
+        sx[3 * at + 1] = d.y[b];
+        sx[3 * at + 2] = d.z[b];
+        sv[3 * at] = d.vx[b] + vs[0];
+        sv[3 * at + 1] = d.vy[b] + vs[1];
+        sv[3 * at + 2] = d.vz[b] + vs[2];
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < n; e += T) {
+        o.ids[base + e] = sid[e];
+        o.m[base + e] = sm[e];
+        o.R[base + e] = sR[e];
+    }
+    for (int e = threadIdx.x; e < 3 * n; e += T) {
+        o.x[3 * base + e] = sx[e];
+        o.v[3 * base + e] = sv[e];
+    }
+    return n;
+}
+
+// Systems of up to kExportOne body slots: one cluster sums the momentum (the segments and
+// the tree of segment_sums and system_total, so the same bits), counts and writes, straight
+// to pinned host memory: one launch in place of a memset, two kernels and two copies.
+// Eight blocks, since one SM stores to the host slowly (1001 bodies: 43 us a call with one block, 36
+// with four), one for the least (10 bodies 30 us, 32 with four).
+constexpr int kExportThreads = 256;
+template <int B>
+__global__ void __cluster_dims__(B) __launch_bounds__(kExportThreads) k_export_one(Dev d, int s, int64_t* count, double* buf) {
+    constexpr int SEGS = kExportOne / kSeg;
+    static_assert(SEGS <= kBodyThreads, "a thread a segment");
+    cg::cluster_group cl = cg::this_cluster();
+    auto sync = [&] {
+        if (B > 1) cl.sync();
+        else __syncthreads();
+    };
+    __shared__ double tmp[3][kExportThreads];
+    __shared__ double part[3][kBodyThreads];   // the segments' sums, of the whole system
+    __shared__ int cnt[B];
+    __shared__ double vs[3];
+    const SysInfo si = d.sys[s];
+    const int tid = threadIdx.x, rank = B > 1 ? (int)cl.block_rank() : 0;
+    // whole segments a block (the last ones may have fewer, or none)
+    const int each = ((int)si.cap / kSeg + B - 1) / B * kSeg, k0 = min((int)si.cap, rank * each);
+    const int per = min((int)si.cap, k0 + each) - k0;
+    int mine = 0;
+    if (tid < kBodyThreads)
+        for (int c = 0; c < 3; c++) part[c][tid] = 0.0;
+    sync();   // (every block's part is clear before anyone writes to it)
+    for (int t0 = 0; t0 < per; t0 += kExportThreads) {
+        const int64_t b = si.off + k0 + t0 + tid;
+        const bool live = t0 + tid < per && d.alive[b] != 0;
+        const double m = live ? d.m[b] : 0.0;
+        tmp[0][tid] = live ? m * d.vx[b] : 0.0;
+        tmp[1][tid] = live ? m * d.vy[b] : 0.0;
+        tmp[2][tid] = live ? m * d.vz[b] : 0.0;
+        mine += __syncthreads_count(live);
+        for (int w = kSeg / 2; w >= 1; w >>= 1) {
+            if (tid % kSeg < w)
+                for (int c = 0; c < 3; c++) tmp[c][tid] += tmp[c][tid + w];
+            __syncthreads();
+        }
+        // thread q of the first 12: segment q / 3 of this tile, component q % 3, to every block
+        if (tid < 3 * kExportThreads / kSeg && t0 + tid / 3 * kSeg < per)
+            for (int r = 0; r < B; r++)
+                *cl.map_shared_rank(&part[tid % 3][(k0 + t0) / kSeg + tid / 3], r) = tmp[tid % 3][tid / 3 * kSeg];
+        __syncthreads();
+    }
+    if (tid < B) *cl.map_shared_rank(&cnt[rank], tid) = mine;
+    sync();
+    for (int w = kBodyThreads / 2; w >= 1; w >>= 1) {
+        if (tid < w)
+            for (int c = 0; c < 3; c++) part[c][tid] += part[c][tid + w];
+        __syncthreads();
+    }
+    if (tid < 3) vs[tid] = part[tid][0] / d.M0s[s];
+    __syncthreads();
+    int64_t base = 0, all = 0;
+    for (int r = 0; r < B; r++) {
+        if (r < rank) base += cnt[r];
+        all += cnt[r];
+    }
+    const ExportView o = export_view(buf, si.cap);
+    for (int t0 = 0; t0 < per; t0 += kExportThreads)
+        base += export_tile<kExportThreads>(d, si, k0 + t0 + tid, t0 + tid < per, vs, base, o);
+    if (rank == 0 && tid == 0) *count = all;
+}
+
+// get_state of a larger system s, first pass: its momentum sum m V over the live
 // bodies, by fixed-order segments (the step's closing-jump partials are free
-// between steps), the total written by the system's last block.
-__global__ void __launch_bounds__(kBodyThreads) k_export_sum(Dev d, int s, double* P, int* counter) {
+// between steps), the total written by the system's last block, and each block's live bodies.
+__global__ void __launch_bounds__(kBodyThreads) k_export_sum(Dev d, int s, double* P, int* counter, int* blocks) {
     const SysInfo si = d.sys[s];
     const int64_t first = si.off + (int64_t)blockIdx.x * kBodyThreads;
     const int64_t b = first + threadIdx.x;
     double px = 0.0, py = 0.0, pz = 0.0;
-    if (d.alive[b]) {
+    const bool live = d.alive[b] != 0;
+    if (live) {
         const double m = d.m[b];
         px = m * d.vx[b];
         py = m * d.vy[b];
         pz = m * d.vz[b];
     }
+    const int n = __syncthreads_count(live);
+    if (threadIdx.x == 0) blocks[blockIdx.x] = n;
     segment_sums(d, first, px, py, pz, d.pP_close);
     system_total(d, d.pP_close, si, s, counter, P, nullptr);
 }
 
-// second pass: one record a body for the host, (x, y, z, heliocentric v =
-// V + P / M0, m, R), and its live flag
-__global__ void __launch_bounds__(kBodyThreads) k_export_write(Dev d, int s, const double* P, double* rec,
-                                                               int* alive) {
+// second pass: each block's live bodies after those of the blocks before it; the last
+// block has the count
+__global__ void __launch_bounds__(kBodyThreads) k_export_write(Dev d, int s, const double* P, const int* blocks,
+                                                               int64_t* count, double* buf) {
+    __shared__ int red[kBodyThreads / 32];
+    __shared__ double vs[3];
     const SysInfo si = d.sys[s];
-    const int64_t k = (int64_t)blockIdx.x * kBodyThreads + threadIdx.x;
-    const int64_t b = si.off + k;
-    const double M0 = d.M0s[s];
-    double* r = rec + 8 * k;
-    r[0] = d.x[b];
-    r[1] = d.y[b];
-    r[2] = d.z[b];
-    r[3] = d.vx[b] + P[0] / M0;
-    r[4] = d.vy[b] + P[1] / M0;
-    r[5] = d.vz[b] + P[2] / M0;
-    r[6] = d.m[b];
-    r[7] = d.R[b];
-    alive[k] = d.alive[b];
+    int before = 0;
+    for (int q = threadIdx.x; q < (int)blockIdx.x; q += kBodyThreads) before += blocks[q];
+    before = __reduce_add_sync(0xffffffffu, before);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = before;
+    if (threadIdx.x < 3) vs[threadIdx.x] = P[threadIdx.x] / d.M0s[s];
+    __syncthreads();
+    before = 0;
+#pragma unroll
+    for (int w = 0; w < kBodyThreads / 32; w++) before += red[w];
+    const int n = export_tile<kBodyThreads>(d, si, (int64_t)blockIdx.x * kBodyThreads + threadIdx.x, true, vs, before,
+                                            export_view(buf, si.cap));
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *count = before + n;
 }
 
 // ---------------------------------------------------------------------------
@@ -694,11 +824,15 @@ void launch_finish(const Dev& d, cudaStream_t s) {
     k_finish<<<152, 256, 0, s>>>(d);
     prof_mark("finish");
 }
-void launch_export(const Dev& d, int sys, int64_t cap, double* P, int* counter, double* rec, int* alive,
+void launch_export_one(const Dev& d, int sys, int64_t cap, int64_t* count, double* buf, cudaStream_t s) {
+    if (cap <= 256) k_export_one<1><<<1, kExportThreads, 0, s>>>(d, sys, count, buf);
+    else k_export_one<8><<<8, kExportThreads, 0, s>>>(d, sys, count, buf);
+}
+void launch_export(const Dev& d, int sys, int64_t cap, double* P, int* counter, int* blocks, int64_t* count, double* buf,
                    cudaStream_t s) {
     const unsigned nb = (unsigned)(cap / kBodyThreads);
-    k_export_sum<<<nb, kBodyThreads, 0, s>>>(d, sys, P, counter);
-    k_export_write<<<nb, kBodyThreads, 0, s>>>(d, sys, P, rec, alive);
+    k_export_sum<<<nb, kBodyThreads, 0, s>>>(d, sys, P, counter, blocks);
+    k_export_write<<<nb, kBodyThreads, 0, s>>>(d, sys, P, blocks, count, buf);
 }
 
 }  // namespace opal

@@ -91,12 +91,11 @@ struct opal_sim {
     int64_t last_inv_big = 0;                // of them big bodies (sources of force)
     int64_t n_big = 0;                       // big bodies of all systems
     cudaEvent_t kick_ev[2] = {nullptr, nullptr};
-    double* d_rec = nullptr;       // get_state: one record of 8 doubles a body, the largest system
-    int* d_ralive = nullptr;       // get_state: live flags
+    double* d_rec = nullptr;       // get_state: 9 doubles a body slot, the largest system of more than kExportOne
+    int* d_exblk = nullptr;        // get_state: live bodies of each block
     double* d_exP = nullptr;       // get_state: the system's momentum
     int* d_excnt = nullptr;        // get_state: blocks done with their segments, a system
-    double* h_rec = nullptr;       // pinned host copies of the two (allocated at the first get_state)
-    int* h_ralive = nullptr;
+    int64_t* h_count = nullptr;    // pinned: the live bodies' count, and the arrays of smaller systems (first get_state)
     double* d_en_body = nullptr;
     float4 *d_en_a = nullptr, *d_en_b = nullptr;   // the energy's float pairs of every body
     double* d_en_pair = nullptr;
@@ -587,10 +586,11 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
     {
         int64_t maxcap = 0;
         for (auto& si : s->sys) maxcap = std::max(maxcap, si.cap);
-        TRYF(dalloc(s, &s->d_rec, 8 * maxcap));
-        TRYF(dalloc(s, &s->d_ralive, maxcap));
+        TRYF(dalloc(s, &s->d_rec, maxcap > kExportOne ? 9 * maxcap : 1));
+        TRYF(dalloc(s, &s->d_exblk, maxcap / kBodyThreads));
         TRYF(dalloc(s, &s->d_exP, 3));
         TRYF(dalloc(s, &s->d_excnt, nsys));
+        CKF(cudaMemsetAsync(s->d_excnt, 0, nsys * sizeof(int), s->stream));
     }
     TRYF(dalloc(s, &s->d_en_body, kEnSums * (N / 128)));
     TRYF(dalloc(s, &s->d_en_a, N));
@@ -1005,30 +1005,31 @@ opal_status opal_get_state(const opal_sim* cs, int32_t sys, int64_t* n_alive, in
     if (!s) return set_err(g_err, "sim is NULL"), OPAL_EINVAL;
     if (sys < 0 || sys >= s->d.nsys) return set_err(s->err, "no system %d", sys), OPAL_EINVAL;
     const SysInfo si = s->sys[sys];
-    const int64_t n = si.n;
-    if (!s->h_rec) {   // pinned staging for the largest system, kept until destroy
-        int64_t maxcap = 0;
-        for (auto& q : s->sys) maxcap = std::max(maxcap, q.cap);
-        CK(cudaHostAlloc(reinterpret_cast<void**>(&s->h_rec), std::max<int64_t>(1, 8 * maxcap) * 8, 0));
-        CK(cudaHostAlloc(reinterpret_cast<void**>(&s->h_ralive), std::max<int64_t>(1, maxcap) * 4, 0));
+    if (!s->h_count) {   // pinned, kept until destroy
+        int64_t slots = 0;
+        for (auto& q : s->sys)
+            if (q.cap <= kExportOne) slots = std::max(slots, q.cap);
+        CK(cudaHostAlloc(reinterpret_cast<void**>(&s->h_count), (2 + 9 * slots) * 8, 0));
     }
-    CK(cudaMemsetAsync(s->d_excnt, 0, s->d.nsys * sizeof(int), s->stream));
-    launch_export(s->d, sys, si.cap, s->d_exP, s->d_excnt, s->d_rec, s->d_ralive, s->stream);
+    const bool one = si.cap <= kExportOne;
+    double* buf = one ? reinterpret_cast<double*>(s->h_count + 2) : s->d_rec;
+    if (one) launch_export_one(s->d, sys, si.cap, s->h_count, buf, s->stream);
+    else launch_export(s->d, sys, si.cap, s->d_exP, s->d_excnt, s->d_exblk, s->h_count, buf, s->stream);
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(s->h_rec, s->d_rec, n * 8 * 8, cudaMemcpyDeviceToHost, s->stream));
-    CK(cudaMemcpyAsync(s->h_ralive, s->d_ralive, n * 4, cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
-    int64_t k = 0;
-    for (int64_t i = 0; i < n; i++) {
-        if (!s->h_ralive[i]) continue;
-        const double* r = s->h_rec + 8 * i;
-        if (ids) ids[k] = i;
-        if (m) m[k] = r[6];
-        if (radius) radius[k] = r[7];
-        if (x) { x[3 * k] = r[0]; x[3 * k + 1] = r[1]; x[3 * k + 2] = r[2]; }
-        if (v) { v[3 * k] = r[3]; v[3 * k + 1] = r[4]; v[3 * k + 2] = r[5]; }
-        k++;
+    const int64_t k = *s->h_count;
+    // the arrays as they lie: from the pinned copy, or from the device straight to the caller
+    const struct {
+        void* to;
+        const double* from;
+        int64_t width;
+    } out[] = {{ids, buf, 1}, {m, buf + si.cap, 1}, {radius, buf + 2 * si.cap, 1}, {x, buf + 3 * si.cap, 3}, {v, buf + 6 * si.cap, 3}};
+    for (auto& o : out) {
+        if (!o.to || k == 0) continue;
+        if (one) std::memcpy(o.to, o.from, o.width * k * 8);
+        else CK(cudaMemcpyAsync(o.to, o.from, o.width * k * 8, cudaMemcpyDeviceToHost, s->stream));
     }
+    if (!one) CK(cudaStreamSynchronize(s->stream));
     if (n_alive) *n_alive = k;
     return OPAL_OK;
 }
@@ -1200,8 +1201,7 @@ void opal_destroy(opal_sim* s) {
     for (auto e : s->kick_ev)
         if (e) cudaEventDestroy(e);
     for (void* p : s->allocs) cudaFree(p);
-    if (s->h_rec) cudaFreeHost(s->h_rec);
-    if (s->h_ralive) cudaFreeHost(s->h_ralive);
+    if (s->h_count) cudaFreeHost(s->h_count);
     if (s->stream) cudaStreamDestroy(s->stream);
     if (s->side) cudaStreamDestroy(s->side);
     if (s->fork_ev) cudaEventDestroy(s->fork_ev);

@@ -27,6 +27,7 @@ constexpr int kBsSoloGroups = 608;  // above this many groups the small-group ke
 constexpr int kBsSoloMid = 76;      // the same for groups of 5-16 members, above this many of them
 constexpr int kBucketDiv = 4;       // body slots per bucket of the spatial sort (cap / 4 buckets a system)
 constexpr int kSmallBodies = 1536;  // body slots up to which one system takes the small-system path
+constexpr int kExportOne = 8192;    // body slots up to which one cluster writes get_state's arrays to the host
 constexpr int kBsOut = 9;           // doubles per member slot of the BS side buffer: x, V, m, R, alive
 constexpr int kFixParts = 4;        // the kick's correction after the encounters: member ranges per body
 constexpr int kBsRows = 8;          // extrapolation rows: n_k = 2, 4, ..., 16
@@ -717,7 +718,9 @@ void launch_energy(const Dev& d, int sys, const SysInfo& si, int nsm, float4* sa
 // get_state of system sys (cap bodies): records (x, y, z, heliocentric v, m, R)
 // and live flags, one a body, into rec and alive; P: 3 doubles of scratch
 // (counter: nsys ints, zero on entry)
-void launch_export(const Dev& d, int sys, int64_t cap, double* P, int* counter, double* rec, int* alive,
+// get_state: the live bodies' ids, m, R, x and v (9 doubles a slot of the system, see export_view) and their count
+void launch_export_one(const Dev& d, int sys, int64_t cap, int64_t* count, double* buf, cudaStream_t s);
+void launch_export(const Dev& d, int sys, int64_t cap, double* P, int* counter, int* blocks, int64_t* count, double* buf,
                    cudaStream_t s);
 void launch_debug_drift(int n, double mu, double dt, int max_iter, double* x, double* v, int* iters, cudaStream_t s);
 void launch_debug_scan_prep(const Dev& d, cudaStream_t s);

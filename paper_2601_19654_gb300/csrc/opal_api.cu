@@ -9,6 +9,7 @@
 #include <cstdlib>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/opal.h"
@@ -521,33 +522,44 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
     TRYF(dalloc(s, &d.gcls, 2 * d.gcap));
     TRYF(dalloc(s, &d.ghard, d.gcap));
     TRYF(dalloc(s, &d.ghuge, d.gcap));
-    // buffers of the whole-GPU encounter kernel, for groups of up to min(N, kHugeMax)
+    // buffers of the whole-GPU encounter kernel, for groups of up to min(N, kHugeMax): one
+    // allocation, none where no group can have more than 64 members
     for (HugeBuf& H : d.hb) {
         H.cap = std::min<int64_t>(N, kHugeMax);   // (a multiple of 32)
-        const int64_t arrays = 2 * kBsRows + 2;
-        TRYF(dalloc(s, &H.pos, arrays * 3 * H.cap));
-        TRYF(dalloc(s, &H.posf, arrays * H.cap));
-        TRYF(dalloc(s, &H.box, 2 * 3 * huge_boxes(H.cap)));
-        TRYF(dalloc(s, &H.mot, 2 * H.cap));
-        TRYF(dalloc(s, &H.list, huge_boxes(H.cap) * kHugeListed));
-        TRYF(dalloc(s, &H.listed, huge_boxes(H.cap)));
-        TRYF(dalloc(s, &H.yv, 2 * 3 * H.cap));
-        TRYF(dalloc(s, &H.zv, (int64_t)kBsRows * 3 * H.cap));
-        TRYF(dalloc(s, &H.z0, (int64_t)kBsRows * 6 * H.cap));
-        TRYF(dalloc(s, &H.row, (int64_t)kBsRows * 6 * H.cap));
-        TRYF(dalloc(s, &H.sk, 6 * H.cap));
-        TRYF(dalloc(s, &H.ska, H.cap));
+        const int64_t arrays = 2 * kBsRows + 2, boxes = huge_boxes(H.cap);
         // blocks' units of a sequence: those of 32 members a warp, or of at most a member a warp of the launch
-        const int64_t units = huge_boxes(H.cap) / kHugeUnitWarps + kHugeTeams * s->nsm + 2;
-        TRYF(dalloc(s, &H.react, (int64_t)2 * kBsRows * units * kHugeWide * 3));
-        TRYF(dalloc(s, &H.m, H.cap));
-        TRYF(dalloc(s, &H.R, H.cap));
-        TRYF(dalloc(s, &H.rc, H.cap));
-        TRYF(dalloc(s, &H.pinv, H.cap));
-        TRYF(dalloc(s, &H.alive, H.cap));
-        TRYF(dalloc(s, &H.gid, H.cap));
-        TRYF(dalloc(s, &H.perm, H.cap));
-        TRYF(dalloc(s, &H.key, H.cap));
+        const int64_t units = boxes / kHugeUnitWarps + kHugeTeams * s->nsm + 2;
+        if (d.nmax <= 64) break;
+        char* base = nullptr;
+        for (int pass = 0; pass < 2; pass++) {   // the size, then the pointers
+            int64_t at = 0;
+            auto part = [&](auto** q, int64_t count) {
+                if (pass) *q = reinterpret_cast<std::remove_reference_t<decltype(*q)>>(base + at);
+                at += (count * (int64_t)sizeof(**q) + 255) / 256 * 256;
+            };
+            part(&H.pos, arrays * 3 * H.cap);
+            part(&H.posf, arrays * H.cap);
+            part(&H.box, 2 * 3 * boxes);
+            part(&H.mot, 2 * H.cap);
+            part(&H.list, boxes * kHugeListed);
+            part(&H.listed, boxes);
+            part(&H.yv, 2 * 3 * H.cap);
+            part(&H.zv, (int64_t)kBsRows * 3 * H.cap);
+            part(&H.z0, (int64_t)kBsRows * 6 * H.cap);
+            part(&H.row, (int64_t)kBsRows * 6 * H.cap);
+            part(&H.sk, 6 * H.cap);
+            part(&H.ska, H.cap);
+            part(&H.react, (int64_t)2 * kBsRows * units * kHugeWide * 3);
+            part(&H.m, H.cap);
+            part(&H.R, H.cap);
+            part(&H.rc, H.cap);
+            part(&H.pinv, H.cap);
+            part(&H.alive, H.cap);
+            part(&H.gid, H.cap);
+            part(&H.perm, H.cap);
+            part(&H.key, H.cap);
+            if (!pass) TRYF(dalloc(s, &base, at));
+        }
     }
     TRYF(dalloc(s, &d.hctl, kHugeTeams));
     CKF(cudaMemsetAsync(d.hctl, 0, kHugeTeams * sizeof(HugeCtl), s->stream));

@@ -152,6 +152,98 @@ __global__ void __launch_bounds__(kBodyThreads) k_sort_count(Dev d) {
     atomicAdd(&d.cstart[key], 1);
 }
 
+// exclusive scan over the block of (members, groups) packed in a long long
+template <int NT>
+__device__ __forceinline__ long long block_excl(long long sum, long long* warp_sum, long long& total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    long long x = sum;
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) warp_sum[warp] = x;
+    __syncthreads();
+    long long before = 0;
+    total = 0;
+#pragma unroll
+    for (int w = 0; w < NT / 32; w++) {
+        const long long ws = warp_sum[w];
+        if (w < warp) before += ws;
+        total += ws;
+    }
+    __syncthreads();
+    return before + x - sum;
+}
+
+// The scans of more than kScanOne counts take two launches of a block for every
+// kScanBlock of them: the blocks' sums, then each block's scan from the sums before it.
+// One block takes 3 us for 16384 counts and as long for each further 16384: 65792 buckets 40
+// to 7 us, 263168 groups' counts 50 to 7.
+constexpr int kScanThreads = 256, kScanPer = 16, kScanBlock = kScanThreads * kScanPer;
+constexpr int64_t kScanOne = 32768;
+
+// 16 counts of a thread (zeros past the end; arrays are padded to whole groups of four)
+__device__ __forceinline__ void load_counts(const int* a, int64_t k0, int64_t n, int (&v)[kScanPer]) {
+#pragma unroll
+    for (int u = 0; u < kScanPer / 4; u++) {
+        const int64_t k = k0 + 4 * u;
+        if (k + 4 <= n) {
+            const int4 q = *reinterpret_cast<const int4*>(a + k);
+            v[4 * u] = q.x; v[4 * u + 1] = q.y; v[4 * u + 2] = q.z; v[4 * u + 3] = q.w;
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; e++) v[4 * u + e] = k + e < n ? a[k + e] : 0;
+        }
+    }
+}
+// low word the counts' sum, high word how many are above zero
+__device__ __forceinline__ long long count_sum(const int (&v)[kScanPer]) {
+    long long s = 0;
+#pragma unroll
+    for (int u = 0; u < kScanPer; u++) s += (long long)v[u] + (v[u] > 0 ? (1LL << 32) : 0LL);
+    return s;
+}
+// the sums of the blocks before this one (every thread of the block calls it)
+__device__ __forceinline__ long long sums_before(const long long* part) {
+    __shared__ long long red[kScanThreads / 32];
+    long long s = 0;
+    for (int q = threadIdx.x; q < (int)blockIdx.x; q += kScanThreads) s += part[q];
+    for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    s = 0;
+#pragma unroll
+    for (int w = 0; w < kScanThreads / 32; w++) s += red[w];
+    return s;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_sums(Dev d, const int* counts, int64_t n, int groups) {
+    if (d.ctl->status || (groups && d.ctl->nflag == 0)) return;
+    __shared__ long long warp_sum[kScanThreads / 32];
+    int v[kScanPer];
+    load_counts(counts, (int64_t)blockIdx.x * kScanBlock + threadIdx.x * kScanPer, n, v);
+    long long total;
+    block_excl<kScanThreads>(count_sum(v), warp_sum, total);
+    if (threadIdx.x == 0) d.scan_part[blockIdx.x] = total;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_sort_prefix_wide(Dev d) {
+    OPAL_TIMELINE_SCOPE(kTlSortPrefix);
+    if (d.ctl->status) return;
+    __shared__ long long warp_sum[kScanThreads / 32];
+    const int64_t k0 = (int64_t)blockIdx.x * kScanBlock + threadIdx.x * kScanPer;
+    int v[kScanPer];
+    load_counts(d.cstart, k0, d.ncell, v);
+    const long long before = sums_before(d.scan_part);
+    long long total;
+    int excl = (int)((before + block_excl<kScanThreads>(count_sum(v), warp_sum, total)) & 0xffffffffLL);
+#pragma unroll
+    for (int u = 0; u < kScanPer; u++) {
+        if (k0 + u < d.ncell) d.ccursor[k0 + u] = excl;
+        excl += v[u];
+    }
+}
+
 // exclusive prefix sum of the bucket counts (one block): each pass, every
 // thread loads 16 consecutive counts at once (vector loads), the block scans
 // the per-thread sums, and a carry runs from pass to pass
@@ -686,6 +778,35 @@ __global__ void __launch_bounds__(1024) k_group_offsets(Dev d) {
     }
 }
 
+// the same by blocks (see k_scan_sums)
+__global__ void __launch_bounds__(kScanThreads) k_group_offsets_wide(Dev d) {
+    OPAL_TIMELINE_SCOPE(kTlGroupOffsets);
+    if (d.ctl->status || d.ctl->nflag == 0) return;
+    __shared__ long long warp_sum[kScanThreads / 32];
+    const int64_t k0 = (int64_t)blockIdx.x * kScanBlock + threadIdx.x * kScanPer;
+    int v[kScanPer];
+    load_counts(d.gcount, k0, d.ntot, v);
+    const long long before = sums_before(d.scan_part);
+    long long total;
+    long long excl = before + block_excl<kScanThreads>(count_sum(v), warp_sum, total);
+#pragma unroll
+    for (int u = 0; u < kScanPer; u++)
+        if (v[u] > 0) {
+            const int gi = (int)(excl >> 32), off = (int)(excl & 0xffffffffLL);
+            d.gofs[k0 + u] = off;
+            d.goff[gi] = off;
+            d.gidx[k0 + u] = gi;
+            excl += (long long)v[u] + (1LL << 32);
+        }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+        const long long all = before + total;
+        const int ng = (int)(all >> 32), nm = (int)(all & 0xffffffffLL);
+        d.goff[ng] = nm;
+        d.ctl->ngroups = ng;
+        d.ctl->ninvolved = nm;
+    }
+}
+
 __global__ void __launch_bounds__(kBodyThreads) k_group_place(Dev d) {
     OPAL_TIMELINE_SCOPE(kTlGroupPlace);
     if (d.ctl->status || d.ctl->nflag == 0) return;
@@ -775,29 +896,6 @@ __global__ void __launch_bounds__(256) k_group_order(Dev d) {
 // The scan and the groups of one small system in one kernel.  (One block for the groups
 // of larger systems was slower than the five kernels: 12 against 9 us at 5003 bodies, 30
 // against 10 at 16384; in shared memory, up to kSmallBodies bodies, it takes 5 in place of 9.)
-
-// exclusive scan over the block of (members, groups) packed in a long long
-template <int NT>
-__device__ __forceinline__ long long block_excl(long long sum, long long* warp_sum, long long& total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    long long x = sum;
-    for (int o = 1; o < 32; o <<= 1) {
-        const long long y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) warp_sum[warp] = x;
-    __syncthreads();
-    long long before = 0;
-    total = 0;
-#pragma unroll
-    for (int w = 0; w < NT / 32; w++) {
-        const long long ws = warp_sum[w];
-        if (w < warp) before += ws;
-        total += ws;
-    }
-    __syncthreads();
-    return before + x - sum;
-}
 
 // ranges ascending, and the groups' lists: a thread a group of up to eight members, the
 // block the larger ones one after another (v: kSmallSlots ints)
@@ -1064,7 +1162,13 @@ void launch_sort_bodies(const Dev& d, cudaStream_t s) {
     const unsigned nb = (unsigned)(d.ntot / kBodyThreads);
     k_sort_count<<<nb, kBodyThreads, 0, s>>>(d);
     prof_mark("scan: sort count");
-    k_sort_prefix<<<1, 1024, 0, s>>>(d);
+    if (d.ncell > kScanOne) {
+        const unsigned blocks = (unsigned)((d.ncell + kScanBlock - 1) / kScanBlock);
+        k_scan_sums<<<blocks, kScanThreads, 0, s>>>(d, d.cstart, d.ncell, 0);
+        k_sort_prefix_wide<<<blocks, kScanThreads, 0, s>>>(d);
+    } else {
+        k_sort_prefix<<<1, 1024, 0, s>>>(d);
+    }
     prof_mark("scan: sort prefix");
     k_sort_scatter<<<nb, kBodyThreads, 0, s>>>(d);
     prof_mark("scan: sort scatter");
@@ -1100,7 +1204,13 @@ void launch_group(const Dev& d, int nsm, cudaStream_t s) {
     prof_mark("group: link");
     k_group_count<<<nb, kBodyThreads, 0, s>>>(d);
     prof_mark("group: count");
-    k_group_offsets<<<1, 1024, 0, s>>>(d);
+    if (d.ntot > kScanOne) {
+        const unsigned blocks = (unsigned)((d.ntot + kScanBlock - 1) / kScanBlock);
+        k_scan_sums<<<blocks, kScanThreads, 0, s>>>(d, d.gcount, d.ntot, 1);
+        k_group_offsets_wide<<<blocks, kScanThreads, 0, s>>>(d);
+    } else {
+        k_group_offsets<<<1, 1024, 0, s>>>(d);
+    }
     prof_mark("group: offsets");
     k_group_place<<<nb, kBodyThreads, 0, s>>>(d);
     prof_mark("group: place");

@@ -490,6 +490,7 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
     TRYF(dalloc(s, &d.kbox, 2 * (N / kKickBox)));
     TRYF(dalloc(s, &d.kbox2, 2 * (N / (2 * kKickBox))));
     d.ncell = (int)(N / kBucketDiv);
+    TRYF(dalloc(s, &d.scan_part, N / 4096 + 1));
     TRYF(dalloc(s, &d.sbox, 6 * nsys));
     TRYF(dalloc(s, &d.ckey, N));
     TRYF(dalloc(s, &d.cstart, d.ncell));

@@ -239,6 +239,7 @@ struct Dev {
     float4* cen_sorted;                 // their midpoint records, in sorted order
     float* tbox;                        // [ntot / 64][6] tile boxes of c +- s
     int ncell;                          // buckets: one per kBucketDiv body slots
+    long long* scan_part;               // sums of the scans' blocks (one for 4096 counts)
     // encounter pipeline
     int* tov;                           // tile pairs whose boxes overlap (indices into the tile list)
     int2* near;  int64_t near_cap;      // pairs passing the midpoint test

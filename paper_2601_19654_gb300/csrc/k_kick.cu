@@ -981,14 +981,21 @@ __global__ void __launch_bounds__(kSmallKickThreads) k_kick_small(Dev d, int nbl
         red[1][tid] = py;
         red[2][tid] = pz;
         __syncthreads();
-        for (int w = kSmallKickThreads / 2; w >= 1; w >>= 1) {
-            if (tid < w)
-                for (int c = 0; c < 3; c++) red[c][tid] += red[c][tid + w];
-            __syncthreads();
-        }
-        if (tid < 3) {
-            d.Ptot[3 * d.nsys + tid] = red[tid][0];
-            d.Pjump[3 * d.nsys + tid] = 0.5 * d.p.dt * red[tid][0] / d.M0s[0];
+        const int c = tid >> 5;   // a warp a component (see segment_sums)
+        if (c < 3) {
+            double v[kSmallKickThreads / 32];
+#pragma unroll
+            for (int w = 0; w < kSmallKickThreads / 32; w++) v[w] = red[c][32 * w + lane];
+#pragma unroll
+            for (int h = kSmallKickThreads / 64; h >= 1; h >>= 1)
+#pragma unroll
+                for (int w = 0; w < h; w++) v[w] += v[w + h];
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) v[0] += __shfl_down_sync(0xffffffffu, v[0], o);
+            if (lane == 0) {
+                d.Ptot[3 * d.nsys + c] = v[0];
+                d.Pjump[3 * d.nsys + c] = 0.5 * d.p.dt * v[0] / d.M0s[0];
+            }
         }
         return;
     }

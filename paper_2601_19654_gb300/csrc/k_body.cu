@@ -514,7 +514,7 @@ __global__ void __cluster_dims__(B) __launch_bounds__(kExportThreads) k_export_o
     __shared__ int cnt[B];
     __shared__ double vs[3];
     const SysInfo si = d.sys[s];
-    const int tid = threadIdx.x, rank = B > 1 ? (int)cl.block_rank() : 0;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rank = B > 1 ? (int)cl.block_rank() : 0;
     // whole segments a block (the last ones may have fewer, or none)
     const int each = ((int)si.cap / kSeg + B - 1) / B * kSeg, k0 = min((int)si.cap, rank * each);
     const int per = min((int)si.cap, k0 + each) - k0;
@@ -530,25 +530,25 @@ __global__ void __cluster_dims__(B) __launch_bounds__(kExportThreads) k_export_o
         tmp[1][tid] = live ? m * d.vy[b] : 0.0;
         tmp[2][tid] = live ? m * d.vz[b] : 0.0;
         mine += __syncthreads_count(live);
-        for (int w = kSeg / 2; w >= 1; w >>= 1) {
-            if (tid % kSeg < w)
-                for (int c = 0; c < 3; c++) tmp[c][tid] += tmp[c][tid + w];
-            __syncthreads();
+        // a warp a segment and component of this tile (see segment_sums), to every block
+        for (int q = warp; q < 3 * kExportThreads / kSeg; q += kExportThreads / 32) {
+            const int c = q % 3, h = q / 3;
+            double v = tmp[c][h * kSeg + lane] + tmp[c][h * kSeg + 32 + lane];
+#pragma unroll
+            for (int w = 16; w >= 1; w >>= 1) v += __shfl_down_sync(0xffffffffu, v, w);
+            v = __shfl_sync(0xffffffffu, v, 0);
+            if (lane < B && t0 + h * kSeg < per) *cl.map_shared_rank(&part[c][(k0 + t0) / kSeg + h], lane) = v;
         }
-        // thread q of the first 12: segment q / 3 of this tile, component q % 3, to every block
-        if (tid < 3 * kExportThreads / kSeg && t0 + tid / 3 * kSeg < per)
-            for (int r = 0; r < B; r++)
-                *cl.map_shared_rank(&part[tid % 3][(k0 + t0) / kSeg + tid / 3], r) = tmp[tid % 3][tid / 3 * kSeg];
         __syncthreads();
     }
     if (tid < B) *cl.map_shared_rank(&cnt[rank], tid) = mine;
     sync();
-    for (int w = kBodyThreads / 2; w >= 1; w >>= 1) {
-        if (tid < w)
-            for (int c = 0; c < 3; c++) part[c][tid] += part[c][tid + w];
-        __syncthreads();
+    if (warp < 3) {   // (see system_total)
+        double v = (part[warp][lane] + part[warp][lane + 64]) + (part[warp][lane + 32] + part[warp][lane + 96]);
+#pragma unroll
+        for (int w = 16; w >= 1; w >>= 1) v += __shfl_down_sync(0xffffffffu, v, w);
+        if (lane == 0) vs[warp] = v / d.M0s[s];
     }
-    if (tid < 3) vs[tid] = part[tid][0] / d.M0s[s];
     __syncthreads();
     int64_t base = 0, all = 0;
     for (int r = 0; r < B; r++) {

@@ -203,9 +203,10 @@ void* opal_stream(const opal_sim* sim);
 opal_status opal_profile_steps(opal_sim* sim, int64_t nsteps, int32_t cap, int32_t* nk,
                                double* ms, const char** names);
 
-/* One line naming the kick kernel variant and launch shape in use (chosen
- * at create by timing the variants on the simulation's own bodies when the
- * pair count makes it worthwhile; OPAL_KICK_VARIANT=<index> forces one). */
+/* One line naming the kick kernel variant and launch shape in use (the mixed
+ * form's chosen at create by timing the variants on the simulation's own bodies when
+ * the pair count makes it worthwhile, the FP64 form's by the sizes;
+ * OPAL_KICK_VARIANT=<index> forces one; one small mixed system takes a kick of its own). */
 const char* opal_kick_config(const opal_sim* sim);
 
 /* Timing of the kick inside the step graph: with enable != 0 the graph is

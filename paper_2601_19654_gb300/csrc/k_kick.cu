@@ -478,43 +478,58 @@ __device__ __forceinline__ KickJ kick_load(const Dev& d, int64_t b, bool in) {
     return r;
 }
 
+// one step of the rotation: a lane's i-body (a) and the j-body it holds (j, body
+// b); m_j K (x_j - x_i) / r^3 into ai, and with SYM the opposite term into aj
+template <bool SYM>
+__device__ __forceinline__ void kick_pair(const Dev& d, const KickJ& a, double rci, const KickJ& j, int64_t b, int form,
+                                          double (&ai)[3], double (&aj)[3]) {
+    const double dx = j.x - a.x, dy = j.y - a.y, dz = j.z - a.z;
+    const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+    double s;
+    if ((unsigned)__double2hiint(r2) <= (unsigned)max(a.rc2h, j.rc2h)) {   // (a NaN is not near)
+        s = slow_pair_d(r2, 1.0, rci, j.rc2h ? d.rc[b] : 0.0, form);
+    } else {
+        double y;
+        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));
+        const double y2 = y * y, e = fma(-r2, y2, 1.0);
+        const double y3 = y2 * y;
+        s = fma(y3 * e, fma(e, 1.875, 1.5), y3);
+    }
+    const double ti = j.m * s;
+    ai[0] = fma(ti, dx, ai[0]);
+    ai[1] = fma(ti, dy, ai[1]);
+    ai[2] = fma(ti, dz, ai[2]);
+    if (SYM) {
+        const double tj = -(a.m * s);
+        aj[0] = fma(tj, dx, aj[0]);
+        aj[1] = fma(tj, dy, aj[1]);
+        aj[2] = fma(tj, dz, aj[2]);
+    }
+}
+
+// the j-bodies (and with SYM their sums) one lane on
+template <bool SYM>
+__device__ __forceinline__ void kick_rotate(KickJ& j, double (&aj)[3]) {
+    const int next = ((threadIdx.x & 31) + 1) & 31;
+    if (SYM)
+        for (int c = 0; c < 3; c++) aj[c] = __shfl_sync(0xffffffffu, aj[c], next);
+    j.x = __shfl_sync(0xffffffffu, j.x, next);
+    j.y = __shfl_sync(0xffffffffu, j.y, next);
+    j.z = __shfl_sync(0xffffffffu, j.z, next);
+    j.m = __shfl_sync(0xffffffffu, j.m, next);
+    j.rc2h = __shfl_sync(0xffffffffu, j.rc2h, next);
+}
+
 // the 32 steps of a warp's i-bodies (a, one a lane) against 32 j-bodies (j, from
-// jb on): sums of m_j K (x_j - x_i) / r^3 into ai, and with SYM the opposite
-// ones into aj (a lane's own j)
+// jb on); with SYM the j-sums end in a lane's own j
 template <bool SYM>
 __device__ __forceinline__ void kick_turn(const Dev& d, const KickJ& a, double rci, KickJ j, int64_t jb, int form,
                                           double (&ai)[3], double (&aj)[3]) {
-    const int lane = threadIdx.x & 31, next = (lane + 1) & 31;
+    const int lane = threadIdx.x & 31;
 #pragma unroll 2
     for (int k = 0; k < 32; k++) {
-        const double dx = j.x - a.x, dy = j.y - a.y, dz = j.z - a.z;
-        const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-        double s;
-        if ((unsigned)__double2hiint(r2) <= (unsigned)max(a.rc2h, j.rc2h)) {   // (a NaN is not near)
-            const int64_t b = jb + ((lane + k) & 31);
-            s = slow_pair_d(r2, 1.0, rci, j.rc2h ? d.rc[b] : 0.0, form);
-        } else {
-            double y;
-            asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));
-            const double y2 = y * y, e = fma(-r2, y2, 1.0);
-            const double y3 = y2 * y;
-            s = fma(y3 * e, fma(e, 1.875, 1.5), y3);
-        }
-        const double ti = j.m * s;
-        ai[0] = fma(ti, dx, ai[0]);
-        ai[1] = fma(ti, dy, ai[1]);
-        ai[2] = fma(ti, dz, ai[2]);
-        if (SYM) {
-            const double tj = -(a.m * s);
-            aj[0] = __shfl_sync(0xffffffffu, fma(tj, dx, aj[0]), next);
-            aj[1] = __shfl_sync(0xffffffffu, fma(tj, dy, aj[1]), next);
-            aj[2] = __shfl_sync(0xffffffffu, fma(tj, dz, aj[2]), next);
-        }
-        j.x = __shfl_sync(0xffffffffu, j.x, next);
-        j.y = __shfl_sync(0xffffffffu, j.y, next);
-        j.z = __shfl_sync(0xffffffffu, j.z, next);
-        j.m = __shfl_sync(0xffffffffu, j.m, next);
-        j.rc2h = __shfl_sync(0xffffffffu, j.rc2h, next);
+        kick_pair<SYM>(d, a, rci, j, jb + ((lane + k) & 31), form, ai, aj);
+        kick_rotate<SYM>(j, aj);
     }
 }
 
@@ -604,6 +619,81 @@ __global__ void __launch_bounds__(32 * W) k_kick_fp64(Dev d, const KickItem* __r
             d.pacc_x[slot] = kick_sj[k];
             d.pacc_y[slot] = kick_sj[w.istep + k];
             d.pacc_z[slot] = kick_sj[2 * w.istep + k];
+        }
+    }
+    queue_done(d);
+}
+
+// The same for few items: kKickSplit warps share an item's 32 steps (warp p
+// starts with the j-bodies rotated by its first step), and their sums are
+// added in shared memory in the order of the warps.
+// A few items leave the pipe idle: what counts is the chain of a warp's steps,
+// about 0.4 us each, and lanes without bodies, two of which met as a near pair
+// (the divide and square root of the changeover in every step).  So eight
+// warps of four steps: kick alone, 10 bodies 25.6 to 9.3 us, 342 bodies 30.8
+// to 13.4, 301 big and 3000 small 77 to 46 (four warps: 10.3, 14.4, 63).
+// fp64_variant says where it is taken: no system there has more than 928 big
+// bodies, so a super-tile is one tile of 32.
+// Steps in which no lane has two bodies are left out, and so is a body's step
+// with itself.
+constexpr int kKickSplit = 8;
+
+__global__ void __launch_bounds__(32 * kKickSplit) k_kick_fp64_split(Dev d, const KickItem* __restrict__ items, int64_t nitems) {
+    OPAL_TIMELINE_SCOPE(kTlKick);
+    if (d.gated && !d.ctl->reprime) return;   // the re-evaluation after a removal, with none
+    constexpr int P = kKickSplit, K = 32 / P;
+    __shared__ double s_sum[P][6][32];        // each warp's sums of the i side (3) and the j side (3)
+    __shared__ int s_item;
+    if (d.ctl->status) return;
+    const int form = d.p.changeover;
+    const int lane = threadIdx.x & 31, p = threadIdx.x >> 5;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_item = atomicAdd(&d.ctl->kick_next, 1);
+        __syncthreads();
+        const int64_t it = s_item;
+        if (it >= nitems) break;
+        const KickItem w = items[it];
+        const SysInfo si = d.sys[w.sys];
+        const bool pairs = w.istep != 0 && w.i0 != w.j0, own = w.istep != 0 && w.i0 == w.j0;
+        const int ni = (int)(w.i1 - w.i0);
+        const bool in = lane < ni;
+        KickJ a = kick_load(d, w.i0 + lane, in);
+        if (!in) a.x = a.y = a.z = -kKickParked;   // far from a parked j: not a near pair
+        const double rci = in ? d.rc[w.i0 + lane] : 0.0;
+        double ai[3] = {0.0, 0.0, 0.0}, aj[3] = {0.0, 0.0, 0.0};
+        for (int64_t jb = w.j0; jb < w.j1; jb += 32) {   // (one turn but for small bodies)
+            const int nj = (int)(w.j1 - jb < 32 ? w.j1 - jb : 32);
+            const int l0 = (lane + K * p) & 31;
+            KickJ j = kick_load(d, jb + l0, l0 < nj);
+            for (int q = 0; q < K; q++) {
+                const int k = K * p + q;
+                if (own && k == 0) {   // zero, or NaN for a body that is not finite
+                    const double z = (j.x - a.x) + (j.y - a.y) + (j.z - a.z);
+                    if (in)
+                        for (int c = 0; c < 3; c++) ai[c] += z;
+                } else if (k < nj || k > 32 - ni) {   // (else lane + k is past nj for each of the ni lanes)
+                    const int64_t b = jb + ((lane + k) & 31);
+                    if (pairs) kick_pair<true>(d, a, rci, j, b, form, ai, aj);
+                    else kick_pair<false>(d, a, rci, j, b, form, ai, aj);
+                }
+                kick_rotate<true>(j, aj);
+            }
+        }
+        for (int c = 0; c < 3; c++) {
+            s_sum[p][c][lane] = ai[c];
+            s_sum[p][3 + c][(lane + K * (p + 1)) & 31] = aj[c];
+        }
+        __syncthreads();
+        const int64_t row = pairs ? (w.i0 - si.off) / w.istep : 0;
+        for (int q = threadIdx.x; q < (pairs ? 192 : 96); q += 32 * P) {
+            const int c = q >> 5;   // 0 to 2: the i side's sums, 3 to 5: the j side's
+            const int64_t body = (c < 3 ? w.i0 : w.j0) + lane;
+            if (body >= (c < 3 ? w.i1 : w.j1)) continue;
+            double sum = s_sum[0][c][lane];
+            for (int k = 1; k < P; k++) sum += s_sum[k][c][lane];
+            double* to = c % 3 == 0 ? d.pacc_x : c % 3 == 1 ? d.pacc_y : d.pacc_z;
+            to[si.slot0 + (c < 3 ? (int64_t)w.chunk : row) * si.cap + (body - si.off)] = sum;
         }
     }
     queue_done(d);
@@ -1107,6 +1197,11 @@ int occ_fp64() {
     return 16 / W;
 }
 
+void launch_fp64_split(const Dev& d, const KickItem* items, int64_t nitems, int grid, cudaStream_t s) {
+    k_kick_fp64_split<<<grid, 32 * kKickSplit, 0, s>>>(d, items, nitems);
+}
+int occ_fp64_split() { return 16 / kKickSplit; }
+
 static const KickVariant kMixed[] = {
     {"mixed t128 i1", 128, 1, launch_mixed<128, 1, 7>, occ_mixed<128, 1, 7>},
     {"mixed t128 i1 6", 128, 1, launch_mixed<128, 1, 6>, occ_mixed<128, 1, 6>},
@@ -1118,6 +1213,7 @@ static const KickVariant kFp64[] = {
     {"fp64 w1", 32, 1, launch_fp64<1>, occ_fp64<1>},
     {"fp64 w2", 64, 1, launch_fp64<2>, occ_fp64<2>},
     {"fp64 w4", 128, 1, launch_fp64<4>, occ_fp64<4>},
+    {"fp64 split", 32 * kKickSplit, 1, launch_fp64_split, occ_fp64_split},   // kFp64Split: chosen by the sizes alone
 };
 
 int kick_num_variants(int precision) {

@@ -262,23 +262,32 @@ void build_kick_items_fp64(opal_sim* s, int W) {
 
 void build_kick_items(opal_sim* s, int precision, int variant, int slots) {
     if (precision == 1) build_kick_items_mixed(s, slots, kick_itile(precision, variant));
-    else build_kick_items_fp64(s, kick_threads(precision, variant) / 32);
+    else build_kick_items_fp64(s, variant == kFp64Split ? 1 : kick_threads(precision, variant) / 32);
 }
 
 // Warps a block of the FP64 kick: as many (4, 2 or 1: tiles of 128, 64 or 32
 // bodies) as leave every SM 16 items, whose last round then idles little
 // (1001 bodies: 33, 53 and 103 us with 1, 2 and 4; 16384: 5.09, 4.99 and 4.94 ms).
+// With few of them eight warps share an item of 32-body tiles
+// (k_kick_fp64_split): up to three tiles an SM and eleven turns of 32 x 32
+// bodies (435 tiles of 900 bodies: 27.4 us against 30.8 with a warp an item, 528
+// of 1001: 33 and 33, 1128 of 1500: 65 and 55; turns: 1639 of 700 big and 2000
+// small bodies 74 and 107, 1778 of 200 and 8000: 88 and 86, 3805: 166 and 158).
 int fp64_variant(const opal_sim* s) {
-    for (int v = kick_num_variants(0) - 1; v > 0; v--) {
-        const int64_t S = kick_threads(0, v);
-        int64_t items = 0;
+    int64_t turns = 0;
+    auto tiles = [&](int64_t S) {
+        int64_t n = 0;
+        turns = 0;
         for (auto& si : s->sys) {
-            const int64_t T = (si.nb + S - 1) / S;
-            items += T * (T + 1) / 2 + (si.nb > 0 ? (si.n - si.nb + S - 1) / S : 0);
+            const int64_t T = (si.nb + S - 1) / S, Ts = (si.n - si.nb + S - 1) / S;
+            n += T * (T + 1) / 2 + (si.nb > 0 ? Ts : 0);
+            turns += T * (T + 1) / 2 + T * Ts;
         }
-        if (items >= 16 * (int64_t)s->nsm) return v;
-    }
-    return 0;
+        return n;
+    };
+    for (int v = kFp64Split - 1; v > 0; v--)
+        if (tiles(kick_threads(0, v)) >= 16 * (int64_t)s->nsm) return v;
+    return tiles(32) <= 3 * (int64_t)s->nsm && turns <= 11 * (int64_t)s->nsm ? kFp64Split : 0;
 }
 
 void build_pair_tiles(opal_sim* s) {
@@ -446,7 +455,7 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
     const int nvar = kick_num_variants(p->precision);
     const char* force = getenv("OPAL_KICK_VARIANT");
     int only = -1;
-    if (force) only = std::max(0, std::min(nvar - 1, atoi(force)));
+    if (force) only = std::max(0, std::min((p->precision == 0 ? kFp64Split : nvar) - 1, atoi(force)));
     else if (p->precision == 0) only = fp64_variant(s);
     std::vector<std::vector<KickItem>> var_items(nvar);
     std::vector<std::vector<SysInfo>> var_sys(nvar);

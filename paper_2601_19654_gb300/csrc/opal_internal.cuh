@@ -697,6 +697,7 @@ void launch_kick(const Dev& d, const KickItem* items, int64_t nitems, int grid, 
 cudaError_t launch_bs_huge(const Dev& d, int nsm, cudaStream_t s);
 void launch_bs_apply(const Dev& d, int nsm, cudaStream_t s);
 void launch_kick_fix(const Dev& d, int nsm, cudaStream_t s);
+constexpr int kFp64Split = 3;   // the FP64 kick's variant for few items (k_kick_fp64_split)
 int kick_num_variants(int precision);
 const char* kick_variant_name(int precision, int variant);
 int kick_occupancy(int precision, int variant);

@@ -69,3 +69,18 @@ def test_fp64_kick_uneven_ensemble():
     for p, rc in zip(parts, rcs):
         _check(a[k:k + len(rc)], p[0], p[1], rc, 0)
         k += len(rc)
+
+
+@pytest.mark.parametrize("n,n_big", [(1, 1), (2, 2), (17, 16), (31, 31), (33, 32), (64, 1), (65, 33), (129, 129),
+                                     (300, 37), (900, 900), (700, 200)])
+def test_fp64_kick_few_items(n, n_big):
+    """Few items: eight warps share an item's steps, steps without a pair left out."""
+    import oracle
+    from paper_2601_19654_gb300 import opal
+    oracle.build()
+    m, x, v, R = _system(n, n_big)
+    rc = oracle.hill_rcrit(1.0, 3.0, m, x)
+    for form in (0, 1):
+        with opal.Simulation(m, x, v, R, precision=0, changeover=form) as sim:
+            assert sim.kick_config.startswith("fp64 split")
+            _check(sim.debug_accel(rc), m, x, rc, form)

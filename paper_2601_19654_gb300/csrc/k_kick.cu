@@ -627,11 +627,13 @@ __global__ void __launch_bounds__(32 * W) k_kick_fp64(Dev d, const KickItem* __r
 // The same for few items: kKickSplit warps share an item's 32 steps (warp p
 // starts with the j-bodies rotated by its first step), and their sums are
 // added in shared memory in the order of the warps.
-// A few items leave the pipe idle: what counts is the chain of a warp's steps,
-// about 0.4 us each, and lanes without bodies, two of which met as a near pair
-// (the divide and square root of the changeover in every step).  So eight
-// warps of four steps: kick alone, 10 bodies 25.6 to 9.3 us, 342 bodies 30.8
-// to 13.4, 301 big and 3000 small 77 to 46 (four warps: 10.3, 14.4, 63).
+// A warp's FP64 instruction holds its quarter of the SM's pipe for 64 cycles, so
+// one warp an SM takes 20 us for the 640 of a turn with three quarters idle; and
+// lanes without bodies met as near pairs (the divide and square root of the
+// changeover in every step).  So eight warps of four steps: kick alone, 10
+// bodies 25.6 to 9.3 us, 342 bodies 30.8 to 13.4, 301 big and 3000 small 77 to
+// 46 (four warps: 10.3, 14.4, 63).  Two steps of a warp at a time (their chains
+// side by side) gave nothing: it is the pipe, not the chain.
 // fp64_variant says where it is taken: no system there has more than 928 big
 // bodies, so a super-tile is one tile of 32.
 // Steps in which no lane has two bodies are left out, and so is a body's step

@@ -1067,7 +1067,7 @@ __global__ void __launch_bounds__(kHugeThreads, 3) k_bs_huge(Dev d, int nsm) {
                         const int A = r == 0 ? kHugeY + ysel : (r & 1) * kBsRows + k;
                         const double* pos = huge_pos(H, A);
                         const double* vel = r == 0 ? H.yv + (int64_t)ysel * 3 * c : H.zv + (int64_t)k * 3 * c;
-                        const int listed = H.listed[u];
+                        const int listed = dense ? -1 : H.listed[u];   // (dense: more units than the lists have room for)
                         if (own) mo = huge_mot(H, kHugeY + ysel)[i];
                         if (own) {
                             pb = huge_posf(H, A)[i];

@@ -72,3 +72,23 @@ def test_one_step_of_a_large_group_against_oracle(make, merges):
     err = np.linalg.norm(a["x"] - osim.x[alive], axis=1) / np.linalg.norm(osim.x[alive], axis=1)
     assert err.max() <= 1e-9, err.max()
     np.testing.assert_allclose(a["m"], osim.m[alive], rtol=1e-14, atol=0)
+
+
+# A dense group alone takes the blocks of both teams, a member a warp in its last rounds
+# (700 and 1000 warps, more than a group with lists ever has); a short step, of few substeps.
+@pytest.mark.parametrize("n", [700, 1000])
+def test_dense_group_of_a_member_a_warp(n):
+    import oracle
+    from paper_2601_19654_gb300 import opal
+    oracle.build()
+    x, v = _cloud(n, n, 1.0, 1.0, 2e-3, 1e-3)
+    s = ic.System(f"dense{n}", np.full(n, 1e-8), x, v, np.full(n, 1e-9), dt=1e-3, nsteps=1)
+    osim = oracle.Sim.from_system(s, scan_prune=1)
+    assert osim.step(1) == oracle.OK
+    assert osim.alive.all()
+    with opal.Simulation.from_system(s, precision=0, encounter_capacity=1 << 20) as sim:
+        sim.step(1)
+        assert sim.stats()["n_groups"] == 1
+        st = sim.state()
+    err = np.linalg.norm(st["x"] - osim.x, axis=1) / np.linalg.norm(osim.x, axis=1)
+    assert err.max() <= 1e-9, err.max()

@@ -144,7 +144,8 @@ opal_status opal_get_state(const opal_sim* sim, int32_t sys, int64_t* n_alive, i
                            double* m, double* x, double* v, double* radius);
 
 /* Total energy E, angular momentum L and momentum P (in democratic
- * heliocentric variables: P = sum m V, barycentric) of system sys, in FP64;
+ * heliocentric variables: P = sum m V, barycentric) of system sys, in FP64
+ * (the pairs' 1 / r is formed to FP64's precision in other units, its sum in FP64);
  * *E_merged_lost is the running sum of the energy removed by mergers, so
  * E + E_merged_lost is the conserved quantity.  Any output may be NULL. */
 opal_status opal_energy_momentum(const opal_sim* sim, int32_t sys, double* E, double L[3],
@@ -160,9 +161,8 @@ opal_status opal_energy_momentum(const opal_sim* sim, int32_t sys, double* E, do
  * must not synchronize the device while steps are in flight (cudaMalloc
  * and cudaFree may synchronize; this call only enqueues three kernels).
  *   n          bodies, 0 <= n <= 131072; a larger n returns OPAL_EINVAL and
- *              launches nothing (the scratch is a fixed 4.3 MB of device
- *              memory: partial sums, and each body's coordinates and mass
- *              split into floats for the pair sum).
+ *              launches nothing (the scratch is a fixed 106 KB of device
+ *              memory for the blocks' sums).
  *   G, M0      as in opal_params (finite, > 0).
  *   m[n], x[3n], v[3n]   masses, heliocentric positions and heliocentric
  *              velocities (row-major n x 3), device memory of the current

@@ -3,7 +3,8 @@
 // is footnote 1 of Sec. 2.1.1):
 //   E = sum 1/2 m |V|^2 - sum G M0 m / |x| + |P|^2 / (2 M0) - sum_{i<j} G m_i m_j / r_ij,
 //   P = sum m V,  L = sum m x x V.
-// FP64 throughout; every partial is summed in a fixed order.
+// Every sum is FP64, in a fixed order.  The pair sum takes 1 / r_ij to FP64's precision from the
+// FP32 and integer pipes (en_recip); everything else is FP64 arithmetic.
 #include <cuda.h>   // driver types only: cuCtxGetCurrent / cuCtxGetId are reached through the runtime
 #include <algorithm>
 #include <cmath>
@@ -15,41 +16,39 @@ namespace opal {
 
 constexpr int kEnThreads = 128;
 constexpr int kEnTile = 128;       // bodies of an i-tile and of a j-tile of the pair sum
-// Blocks of the pair sum an SM holds: 4 (127 registers) with two pairs under way a thread
-// 0.527 ms at 16384 bodies; 3: 0.548, 5: 0.539, 6: 0.541;
-// one pair at a time 0.544 to 0.561, four 0.538.
-constexpr int kEnBlocks = 4;
+// Blocks of the pair sum an SM holds: 6 (78 registers) 0.729 ms at 16384 bodies and 43.3 at 131072;
+// 3: 0.782 and 46.8, 4: 0.759 and 45.7, 5: 0.740 and 44.2.
+constexpr int kEnBlocks = 6;
 constexpr int kEnShortRun = 32;    // sources of a unit when there are few tiles
 
 // ---------------------------------------------------------------------------
 // Pair potential, sum_{i<j} m_i m_j / r_ij, of n bodies.
 //
-// On this chip FP64 runs at 1/62 of the FP32 rate (measured: 1.25 against 78
-// TFLOP/s), so the sum in plain FP64 (about 20 FP64 instructions a pair with
-// the square root and the division) was bound by the FP64 pipe: 6.1 ms at
-// 16384 bodies and 765 ms at 131072.  From kEnSplitMin bodies on a pair's
-// term is formed in pairs of floats instead (hi + lo; every product's and
-// sum's rounding error is taken along by an FMA or Knuth's TwoSum), about 100
-// FP32 instructions, which the FP32 pipe bounds.  A term is then right to about
-// 2^-47 of itself, independently from pair to pair:
-//  - coordinates and masses are split into three floats, which hold a double
-//    exactly (a body's own rounding would be in all its pairs);
-//  - pairs closer than 1/128 of the i-body's distance take the FP64
-//    expression, and so do pairs with more than 2^-12 of the sum (by its lower
-//    bound (sum m_i m_j)^2 / sum m_i m_j (|x_i| + |x_j|), as r_ij <= |x_i| +
-//    |x_j|), so the errors of the others average: 2^-47 * 2^-6 of the sum at
-//    most, less with more pairs;
-//  - terms about as small as a rounding join a sum before it is rounded (as
-//    the addend of an FMA): added to a rounded float they would be lost
-//    whatever their sign, and the sum over the pairs biased.
-// Measured against the sum of FP64 terms added without rounding, 512 to 131072
-// bodies: both forms within 4e-16 of it, and at 131072 bodies with two giants
-// this one 4e-16, the FP64 one 1.3e-15.  16384 bodies: 6.1 to 0.53 ms; 131072:
-// 765 to 29.7 ms (2.9e11 pairs/s; the 110 instructions of a pair at the FP32
-// pipe's full rate would take 25 ms).  Below 512 bodies the errors have too
-// few pairs to average over, and the sum stays in FP64.  Bodies whose coordinates or masses leave the range in which no part of a float
-// pair under- or overflows take FP64 too, tile by tile, so any units work.
-constexpr int64_t kEnSplitMin = 512;
+// On this chip FP64 runs at 1/62 of the FP32 rate (measured: 1.25 against 78 TFLOP/s): a warp's FP64
+// instruction takes its scheduler 64 cycles.  A pair in plain FP64 with the square root and the
+// division is about 20 of them, with the hardware's approximate reciprocal square root 13.  Here 1 / r
+// is formed as a double by about 133 FP32 operations (two pairs a packed instruction) and 20 integer ones, and
+// one FP64 FMA adds m_j / r to the thread's sum beside them.  Plain FP64: 16384 bodies 6.1 ms, 131072 bodies 765
+// (each pair from both sides); the 13 instructions at the pipe's rate 2.8 and 178; so 0.73 and 43.3 (the packed
+// pipe busy 0.7 of the time; unpacked 0.77 and 46.0).  Pairs of floats (0.53 and 29.7) kept 47 bits of a term.
+//
+// The FP32 part, for bodies of two tiles whose coordinates lie below X, a power of two (everything
+// in units of X, so any units of length work):
+//  - a coordinate is three floats a + b + c, a a multiple of 2^-22, b of 2^-45, c the rest, so that the
+//    differences of the a's and of the b's are exact (those of the c's to 2^-70); their sum by one
+//    FastTwoSum is D1 + D2, |D2| <= half an ulp of D1;
+//  - y = the approximate 1 / r of D1 alone, off by 2^-21.6 at most; with v = y (D1 + D2 + D3), a unit
+//    vector but for y's error, 1 / r = y (1 - d)^(-1/2), d = 1 - v.v, |d| < 2^-20;
+//  - v's components are cut into V (a multiple of 2^-11), A (of 2^-21), B1 (of 2^-31) and C, so that 1 -
+//    V.V - 2 V.A - A.A - 2 V.B1, nearly all of which cancels, is exact in FP32 (multiples of 2^-42, the
+//    partial results below 2^-18 from A.A on); the rest of d, 2 V.C + 2 A.B + B.B, is below 2^-29, in floats;
+//  - 1 / r = y (1 + d/2 + 3/8 d^2) (the next term is below 2^-61) as the 53-bit mantissa of
+//    a double: y's 24 bits and, 29 places lower, y (d/2 + 3/8 d^2), a product of integers rounded once.
+// Error of 1 / r against 113-bit arithmetic, 200000 pairs for each power of two of r from X down to
+// 2^-12 X: 0.52 to 0.53 x 2^-53 rms and 2.7 x 2^-53 at most, mean below 0.002 x 2^-53 (1 / sqrt of the
+// FP64 square: 0.69 to 0.72, 2.8 and 0.003).
+// A pair closer than 2^-12 X takes the FP64 expression, and so do tiles whose coordinates leave
+// the range of the scaling (or are not finite).
 
 // FP64 arrays of the bodies, component c of body i at c[i * stride]; alive may be null
 struct EnSrc {
@@ -58,138 +57,143 @@ struct EnSrc {
     int stride;
 };
 
-// the float pairs of one body: a = hi of x, y, z, m; b = lo.  a.x is a NaN when
-// the body is out of the range of the float form.
-__device__ __forceinline__ void en_split(double x, double y, double z, double m, float4& a, float4& b) {
-    split_hl(x, a.x, b.x);
-    split_hl(y, a.y, b.y);
-    split_hl(z, a.z, b.z);
-    split_hl(m, a.w, b.w);
-    const float big = fmaxf(fabsf(a.x), fmaxf(fabsf(a.y), fabsf(a.z)));
-    const bool ok = big > 0x1p-30f && big < 0x1p30f && (a.w == 0.0f || (a.w > 0x1p-50f && a.w < 0x1p50f)) &&
-                    isfinite(x) && isfinite(y) && isfinite(z) && isfinite(m) && (m == 0.0 || a.w != 0.0f);
-    if (!ok) a.x = __int_as_float(0x7fffffff);
-}
-
-// a + b = s + e exactly
-__device__ __forceinline__ void en_two_sum(float a, float b, float& s, float& e) {
-    s = __fadd_rn(a, b);
-    const float v = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v));
-}
-
-// One unit: body i (this thread's; a, b its float pairs, li its index in the
-// tile) against nj staged sources, those with index above its own when the
-// tiles are the same (diag).  The sum of m_j / r_ij comes back in FP64.
-// `wide`: a body of the unit is out of the float range (or there are few
-// bodies): FP64.
+// the sources of a unit: a, b and c of x, y, z (component 3 q + k), and the FP64 values
 struct EnTile {
-    float4 a[kEnTile], b[kEnTile], c[kEnTile];   // first, second and third floats of x, y, z, m
-    double x[kEnTile], y[kEnTile], z[kEnTile], m[kEnTile];
+    float part[9][kEnTile];
+    double m[kEnTile], x[kEnTile], y[kEnTile], z[kEnTile];
 };
 
-// what two floats leave of a double (exact)
-__device__ __forceinline__ float en_third(double v, float a, float b) { return (float)(v - (double)a - (double)b); }
+// scale: 1 / X
+__device__ __forceinline__ void en_split(double v, double scale, float& a, float& b, float& c) {
+    const double s = v * scale, kA = 0x1.8p30, kB = 0x1.8p7;   // (ulps 2^-22 and 2^-45)
+    const double da = (s + kA) - kA, rest = s - da, db = (rest + kB) - kB;
+    a = trunc_f(da);   // (exact, and so is b)
+    b = trunc_f(db);
+    c = trunc_f(rest - db);
+}
 
+// 1 / |j - i| of two sources j (j2: their nine floats; n: i's, negated), a packed instruction for both where there
+// is one.  Not good (the result means nothing): a separation below 2^-12, zero included, or 1 / r on
+// the other side of a power of two than y, where a mantissa's unit is another (one pair in some 10^6).
+__device__ __forceinline__ void en_recip(const float (&n)[9], const float2 (&j2)[9], double (&out)[2], bool (&good)[2]) {
+    auto all = [](float v) { return make_float2(v, v); };
+    auto sub = [&](float2 a, float2 b) { return __ffma2_rn(b, all(-1.0f), a); };
+    auto cut = [&](float2 a, float k) { return __fadd2_rn(__fadd2_rn(a, all(k)), all(-k)); };   // to a multiple of k's ulp
+    auto dot = [](const float2 (&a)[3], const float2 (&b)[3], float2 c) {
+        return __ffma2_rn(a[2], b[2], __ffma2_rn(a[1], b[1], __ffma2_rn(a[0], b[0], c)));
+    };
+    float2 D1[3], D2[3], V[3], A[3], B[3], C[3], b1[3];
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const float2 p = __fadd2_rn(j2[k], all(n[k])), q = __fadd2_rn(j2[3 + k], all(n[3 + k]));
+        D1[k] = __fadd2_rn(p, q);
+        D2[k] = sub(q, sub(D1[k], p));
+    }
+    const float2 r2 = __ffma2_rn(D1[2], D1[2], __ffma2_rn(D1[1], D1[1], __fmul2_rn(D1[0], D1[0])));
+    float2 y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y.x) : "f"(r2.x));
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y.y) : "f"(r2.y));
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        // v = P + pe + Q + s, the first three exact
+        const float2 P = __fmul2_rn(y, D1[k]), pe = __ffma2_rn(y, D1[k], make_float2(-P.x, -P.y)), Q = __fmul2_rn(y, D2[k]);
+        const float2 s = __ffma2_rn(y, __fadd2_rn(j2[6 + k], all(n[6 + k])), __ffma2_rn(y, D2[k], make_float2(-Q.x, -Q.y)));
+        V[k] = cut(P, 0x1.8p12f);
+        const float2 f = sub(P, V[k]);
+        A[k] = cut(f, 0x1.8p2f);
+        const float2 f2 = sub(f, A[k]);
+        const float2 g = __fadd2_rn(pe, Q), gv = sub(g, pe);
+        const float2 ge = __fadd2_rn(sub(pe, sub(g, gv)), sub(Q, gv));   // g + ge = pe + Q
+        b1[k] = cut(__fadd2_rn(f2, g), 0x1.8p-8f);
+        C[k] = __fadd2_rn(__fadd2_rn(sub(f2, b1[k]), g), __fadd2_rn(ge, s));
+        B[k] = __fadd2_rn(b1[k], C[k]);
+    }
+    const float2 zero = all(0.0f), two = all(2.0f);
+    float2 h = dot(V, V, all(-1.0f));                        // -d = h + l
+    h = __ffma2_rn(two, dot(V, A, zero), h);
+    h = dot(A, A, h);
+    h = __ffma2_rn(two, dot(V, b1, zero), h);
+    const float2 l = dot(B, B, __fmul2_rn(two, dot(A, B, dot(V, C, zero))));
+    // d/2 as h/2 in units of 2^-52 (h is an integer of 22 bits in units of 2^-42, taken from the
+    // low bits of its sum with 1.5 x 2^23) and l/2 - 3/8 d^2 in units of 2^-54, both negative
+    const float2 d = __fadd2_rn(h, l);
+    const float2 hm = __ffma2_rn(h, all(0x1p42f), all(0x1.8p23f));
+    const float2 lm = __ffma2_rn(__fmul2_rn(d, d), all(-0x1.8p52f), __fmul2_rn(l, all(0x1p53f)));
+#pragma unroll
+    for (int e = 0; e < 2; e++) {
+        const int ch = (int)((__float_as_uint(e ? hm.y : hm.x) << 9) ^ 0x80000000u), cl = __float2int_rn(e ? lm.y : lm.x);
+        const unsigned yb = __float_as_uint(e ? y.y : y.x);
+        const int Y = (int)((yb & 0x7fffffu) | 0x800000u);
+        const long long z = ((long long)Y * ch + (long long)(Y >> 2) * cl + (1 << 22)) >> 23;
+        const long long y64 = ((long long)yb << 29) + (896LL << 52), u = y64 - z;
+        good[e] = (e ? r2.y : r2.x) >= 0x1p-24f && (u ^ y64) >> 52 == 0;
+        out[e] = __longlong_as_double(u);
+    }
+}
+
+// the pair's term in FP64 (out of line: few pairs take it)
+__device__ __noinline__ double en_term(const EnTile& T, int jj, double xi, double yi, double zi) {
+    if (T.m[jj] == 0.0) return 0.0;
+    const double fx = T.x[jj] - xi, fy = T.y[jj] - yi, fz = T.z[jj] - zi;
+    return T.m[jj] / sqrt(fx * fx + fy * fy + fz * fz);
+}
+
+// One unit: body i (this thread's) against nj staged sources, those with index above its own
+// when the tiles are the same (DIAG); the sum of m_j / r_ij.
 template <bool DIAG>
-__device__ __forceinline__ double en_unit_split(const EnTile& T, int nj, int first, float4 a, float4 b, double xi,
-                                                double yi, double zi, float most) {
-    const float big = fmaxf(fabsf(a.x), fmaxf(fabsf(a.y), fabsf(a.z)));
-    const float thr = big * big * 0x1p-14f;   // nearer than 1/128 of the largest coordinate: FP64
-    const float ax = en_third(xi, a.x, b.x), ay = en_third(yi, a.y, b.y), az = en_third(zi, a.z, b.z);
-    float sh = 0.0f, sl = 0.0f;
-    double e = 0.0;
-#pragma unroll 2
-    for (int jj = 0; jj < nj; jj++) {
-        const float4 c = T.a[jj], g = T.b[jj], k = T.c[jj];
-        float dx, dy, dz, ex, ey, ez, t;
-        en_two_sum(c.x, -a.x, dx, ex);
-        en_two_sum(c.y, -a.y, dy, ey);
-        en_two_sum(c.z, -a.z, dz, ez);
-        ex = __fadd_rn(__fadd_rn(ex, __fsub_rn(g.x, b.x)), __fsub_rn(k.x, ax));
-        ey = __fadd_rn(__fadd_rn(ey, __fsub_rn(g.y, b.y)), __fsub_rn(k.y, ay));
-        ez = __fadd_rn(__fadd_rn(ez, __fsub_rn(g.z, b.z)), __fsub_rn(k.z, az));
-        t = __fadd_rn(dx, ex); ex = __fsub_rn(ex, __fsub_rn(t, dx)); dx = t;
-        t = __fadd_rn(dy, ey); ey = __fsub_rn(ey, __fsub_rn(t, dy)); dy = t;
-        t = __fadd_rn(dz, ez); ez = __fsub_rn(ez, __fsub_rn(t, dz)); dz = t;
-        // r^2 = rh + rl, rl = 2 (dx ex + ...) + (ex^2 + ...) and the roundings
-        const float px = __fmul_rn(dx, dx), py = __fmul_rn(dy, dy), pz = __fmul_rn(dz, dz);
-        const float qx = __fmaf_rn(dx, dx, -px), qy = __fmaf_rn(dy, dy, -py), qz = __fmaf_rn(dz, dz, -pz);
-        float et, rh, er;
-        en_two_sum(px, py, t, et);
-        en_two_sum(t, pz, rh, er);
-        const float sq = __fmaf_rn(ez, ez, __fmaf_rn(ey, ey, __fmul_rn(ex, ex)));
-        const float cr = __fmaf_rn(dz, ez, __fmaf_rn(dy, ey, __fmaf_rn(dx, ex, __fmul_rn(0.5f, sq))));
-        const float rl =
-            __fmaf_rn(2.0f, cr, __fadd_rn(__fadd_rn(__fadd_rn(qx, qy), qz), __fadd_rn(et, er)));
-        // m y (1 + d/2 + 3/8 d^2), d = 1 - r^2 y^2: the next term is below 2^-66
-        float y;
-        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(rh));
-        const float yh = __fmul_rn(y, y), yl = __fmaf_rn(y, y, -yh);
-        float d = __fmaf_rn(-rh, yh, 1.0f);
-        d = __fmaf_rn(-rh, yl, d);
-        d = __fmaf_rn(-rl, yh, d);
-        float wh = __fmul_rn(c.w, y), wl = __fmaf_rn(c.w, y, -wh);
-        wl = __fadd_rn(wl, __fmaf_rn(g.w, y, __fmul_rn(k.w, y)));
-        wl = __fadd_rn(wl, __fmaf_rn(wh, __fmul_rn(0.5f, d), __fmul_rn(wh, __fmul_rn(__fmul_rn(0.375f, d), d))));
-        // (r = 0 makes y infinite: the tests below take such a pair out before its NaN is added)
-        const bool own = DIAG && first + jj <= (int)threadIdx.x;   // another thread's pair, or the body itself
-        const bool fp64 = (rh < thr || wh > most) && !own;
-        if (fp64 || own) wh = wl = 0.0f;
-        float s, es;
-        en_two_sum(sh, wh, s, es);
-        sh = s;
-        sl = __fadd_rn(sl, __fadd_rn(es, wl));
-        if (fp64 && T.m[jj] != 0.0) {
-            const double fx = T.x[jj] - xi, fy = T.y[jj] - yi, fz = T.z[jj] - zi;
-            e += T.m[jj] / sqrt(fx * fx + fy * fy + fz * fz);
+__device__ __forceinline__ double en_unit(const EnTile& T, int nj, int first, double scale, double xi, double yi, double zi) {
+    float n[9];
+    en_split(-xi, scale, n[0], n[3], n[6]);
+    en_split(-yi, scale, n[1], n[4], n[7]);
+    en_split(-zi, scale, n[2], n[5], n[8]);
+    double e = 0.0, near = 0.0;
+#pragma unroll 1
+    for (int jj = 0; jj < nj; jj += 2) {
+        float2 j2[9];
+#pragma unroll
+        for (int q = 0; q < 9; q++) j2[q] = *reinterpret_cast<const float2*>(&T.part[q][jj]);
+        const double2 m = *reinterpret_cast<const double2*>(&T.m[jj]);
+        double s[2];
+        bool good[2];
+        en_recip(n, j2, s, good);
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            const bool own = DIAG && first + jj + k <= (int)threadIdx.x;   // another thread's pair, or the body itself
+            if (good[k]) e = fma(own ? 0.0 : k ? m.y : m.x, s[k], e);
+            else if (!own) near += en_term(T, jj + k, xi, yi, zi);
         }
     }
-    return e + ((double)sh + (double)sl);
+    return fma(e, scale, near);
 }
 
 __device__ __forceinline__ double en_unit_wide(const EnTile& T, int nj, int from, double xi, double yi, double zi) {
     double e = 0.0;
-    for (int jj = from; jj < nj; jj++) {
-        if (T.m[jj] == 0.0) continue;
-        const double fx = T.x[jj] - xi, fy = T.y[jj] - yi, fz = T.z[jj] - zi;
-        e += T.m[jj] / sqrt(fx * fx + fy * fy + fz * fz);
-    }
+    for (int jj = from; jj < nj; jj++) e += en_term(T, jj, xi, yi, zi);
     return e;
 }
 
-// The pair sum of n bodies from off on (sa, sb their float pairs).  A unit is
-// an i-tile against a run of `run` sources (a whole j-tile, or a quarter of
-// one when there are few) of a j-tile at or above it; block b takes units b,
-// b + gridDim.x, ..., so that the order of every sum is fixed, and its total
-// goes to out[b].  rows: the body kernel's rows (row_n doubles each) of these
-// bodies, from column c0 on the sums of m, m^2 and m |x|.
-__global__ void __launch_bounds__(kEnThreads, kEnBlocks) k_energy_pairs(int64_t n, int64_t off, EnSrc src,
-                                                             const float4* __restrict__ sa,
-                                                             const float4* __restrict__ sb, int run,
-                                                             const double* __restrict__ rows, int row_n, int c0,
-                                                             double* __restrict__ out) {
-    __shared__ EnTile T;
-    __shared__ double red[3][kEnThreads];
+// The pair sum of n bodies from off on.  A unit is an i-tile against a run of `run` sources (a whole
+// j-tile, or a quarter of one when there are few) of a j-tile at or above it; block b takes units b,
+// b + gridDim.x, ..., so that the order of every sum is fixed, and its total goes to out[b].
+__global__ void __launch_bounds__(kEnThreads, kEnBlocks) k_energy_pairs(int64_t n, int64_t off, EnSrc src, int run,
+                                                                     double* __restrict__ out) {
+    __shared__ __align__(16) EnTile T;
+    __shared__ double red[kEnThreads];
+    __shared__ int top[kEnThreads / 32];
     const int64_t nt = (n + kEnTile - 1) / kEnTile;
     const int parts = kEnTile / run;
     const int64_t units = nt * (nt + 1) / 2 * parts;
-    const bool few = n < kEnSplitMin;
-    double most = 0.0;   // m_i times a term's limit in float form
-    if (!few) {
-        double v[3] = {0.0, 0.0, 0.0};
-        for (int64_t b = threadIdx.x; b < nt; b += kEnThreads)
-            for (int c = 0; c < 3; c++) v[c] += rows[b * row_n + c0 + c];
-        for (int c = 0; c < 3; c++) red[c][threadIdx.x] = v[c];
-        __syncthreads();
-        for (int w = kEnThreads / 2; w >= 1; w >>= 1) {
-            if (threadIdx.x < w)
-                for (int c = 0; c < 3; c++) red[c][threadIdx.x] += red[c][threadIdx.x + w];
-            __syncthreads();
-        }
-        const double mm = red[0][0] * red[0][0] - red[1][0];
-        most = 0x1p-12 * mm / (2.0 * red[0][0]) * (0.5 * mm / red[2][0]);
-    }
+    // a body (a massless one adds nothing wherever it is, and is put at the origin), and the
+    // high word of its largest coordinate
+    auto load = [&](int64_t k, double& x, double& y, double& z, double& m) {
+        const int64_t g = off + k, s = g * src.stride;
+        m = src.alive && !src.alive[g] ? 0.0 : src.m[g];
+        const bool any = m != 0.0;
+        x = any ? src.x[s] : 0.0;
+        y = any ? src.y[s] : 0.0;
+        z = any ? src.z[s] : 0.0;
+        return max(__double2hiint(fabs(x)), max(__double2hiint(fabs(y)), __double2hiint(fabs(z))));
+    };
     double total = 0.0;
     for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
         const int64_t w = u / parts;
@@ -202,52 +206,44 @@ __global__ void __launch_bounds__(kEnThreads, kEnBlocks) k_energy_pairs(int64_t 
         const int64_t j0 = B * kEnTile + first, i = A * kEnTile + threadIdx.x;
         const int nj = (int)(n - j0 < run ? n - j0 : run);
         if (nj <= 0) continue;   // (the same for the whole block)
+        double xj = 0.0, yj = 0.0, zj = 0.0, mj = 0.0, xi = 0.0, yi = 0.0, zi = 0.0, mi = 0.0;
+        int hi = 0;
+        if ((int)threadIdx.x < nj) hi = load(j0 + threadIdx.x, xj, yj, zj, mj);
+        if (i < n) hi = max(hi, load(i, xi, yi, zi, mi));
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        __syncthreads();   // (the unit before this one is done with the tile)
+        if ((threadIdx.x & 31) == 0) top[threadIdx.x >> 5] = hi;
         __syncthreads();
-        bool wide = few;
-        if ((int)threadIdx.x < nj) {
-            const int64_t g = off + j0 + threadIdx.x, s = g * src.stride;
-            const float4 a = sa[g], b = sb[g];
-            const double x = src.x[s], y = src.y[s], z = src.z[s];
-            const double m = src.alive && !src.alive[g] ? 0.0 : src.m[g];
-            T.a[threadIdx.x] = a;
-            T.b[threadIdx.x] = b;
-            T.c[threadIdx.x] =
-                make_float4(en_third(x, a.x, b.x), en_third(y, a.y, b.y), en_third(z, a.z, b.z), en_third(m, a.w, b.w));
-            T.x[threadIdx.x] = x;
-            T.y[threadIdx.x] = y;
-            T.z[threadIdx.x] = z;
-            T.m[threadIdx.x] = m;
-            wide |= isnan(a.x);
+#pragma unroll
+        for (int q = 0; q < kEnThreads / 32; q++) hi = max(hi, top[q]);
+        const int k = hi >> 20;                          // coordinates below X = 2^(k - 1022)
+        const bool wide = k < 64 || k > 1983;            // (no scaling: FP64)
+        const double scale = __hiloint2double((2045 - k) << 20, 0);
+        if ((int)threadIdx.x < (nj + 1) / 2 * 2) {   // (a last one without mass where nj is odd)
+            const int t = threadIdx.x;
+            T.x[t] = xj;
+            T.y[t] = yj;
+            T.z[t] = zj;
+            T.m[t] = mj;
+            en_split(xj, scale, T.part[0][t], T.part[3][t], T.part[6][t]);
+            en_split(yj, scale, T.part[1][t], T.part[4][t], T.part[7][t]);
+            en_split(zj, scale, T.part[2][t], T.part[5][t], T.part[8][t]);
         }
-        float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
-        double xi = 0.0, yi = 0.0, zi = 0.0, mi = 0.0;
-        if (i < n) {
-            const int64_t g = off + i, s = g * src.stride;
-            a = sa[g];
-            b = sb[g];
-            xi = src.x[s];
-            yi = src.y[s];
-            zi = src.z[s];
-            mi = src.alive && !src.alive[g] ? 0.0 : src.m[g];
-            wide |= isnan(a.x);
-        }
-        wide = __syncthreads_or(wide);
+        __syncthreads();
         if (mi == 0.0) continue;   // (no barrier between here and the next unit's first)
-        const float lim = (float)(most / mi);
         double e;
         if (wide) e = en_unit_wide(T, nj, A == B ? max(0, (int)threadIdx.x + 1 - first) : 0, xi, yi, zi);
-        else if (A == B) e = en_unit_split<true>(T, nj, first, a, b, xi, yi, zi, lim);
-        else e = en_unit_split<false>(T, nj, first, a, b, xi, yi, zi, lim);
+        else if (A == B) e = en_unit<true>(T, nj, first, scale, xi, yi, zi);
+        else e = en_unit<false>(T, nj, first, scale, xi, yi, zi);
         total += mi * e;
     }
-    __syncthreads();
-    red[0][threadIdx.x] = total;
+    red[threadIdx.x] = total;
     __syncthreads();
     for (int w = kEnThreads / 2; w >= 1; w >>= 1) {
-        if (threadIdx.x < w) red[0][threadIdx.x] += red[0][threadIdx.x + w];
+        if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
         __syncthreads();
     }
-    if (threadIdx.x == 0) out[blockIdx.x] = red[0][0];
+    if (threadIdx.x == 0) out[blockIdx.x] = red[0];
 }
 
 // grid and run length of the pair sum of n bodies: whole j-tiles once they
@@ -259,33 +255,20 @@ static void en_shape(int64_t n, int nsm, int& grid, int& run) {
     grid = (int)std::max<int64_t>(1, std::min<int64_t>(tiles * (kEnTile / run), most));
 }
 
-// body terms of one system from off on: per 128-body block, kEnSums sums (kinetic +
-// central, P, L, then m, m^2 and m |x|), and the float pairs of its bodies for the pair sum
-__global__ void __launch_bounds__(kEnThreads) k_energy_body(Dev d, int64_t off, double* body_part, float4* sa,
-                                                            float4* sb) {
+// body terms of one system from off on: per 128-body block, kEnSums sums (kinetic + central, P, L)
+__global__ void __launch_bounds__(kEnThreads) k_energy_body(Dev d, int64_t off, double* body_part) {
     __shared__ double red[kEnSums][kEnThreads];
     const int64_t b = off + (int64_t)blockIdx.x * kEnThreads + threadIdx.x;
     double v[kEnSums] = {};
-    const double x = d.x[b], y = d.y[b], z = d.z[b];
-    const bool alive = d.alive[b] != 0;
-    const double m = alive ? d.m[b] : 0.0;
-    float4 fa, fb;
-    en_split(x, y, z, m, fa, fb);
-    sa[b] = fa;
-    sb[b] = fb;
-    if (alive) {
-        const double vx = d.vx[b], vy = d.vy[b], vz = d.vz[b];
-        const double r = sqrt(x * x + y * y + z * z);
-        v[0] = 0.5 * m * (vx * vx + vy * vy + vz * vz) - d.p.G * d.M0s[d.body_sys[b]] * m / r;
+    if (d.alive[b]) {
+        const double m = d.m[b], x = d.x[b], y = d.y[b], z = d.z[b], vx = d.vx[b], vy = d.vy[b], vz = d.vz[b];
+        v[0] = 0.5 * m * (vx * vx + vy * vy + vz * vz) - d.p.G * d.M0s[d.body_sys[b]] * m / sqrt(x * x + y * y + z * z);
         v[1] = m * vx;
         v[2] = m * vy;
         v[3] = m * vz;
         v[4] = m * (y * vz - z * vy);
         v[5] = m * (z * vx - x * vz);
         v[6] = m * (x * vy - y * vx);
-        v[7] = m;
-        v[8] = m * m;
-        v[9] = m * r;
     }
     for (int c = 0; c < kEnSums; c++) red[c][threadIdx.x] = v[c];
     __syncthreads();
@@ -303,7 +286,7 @@ __global__ void k_energy_final(Dev d, int s, int64_t nb, int np, const double* b
     __shared__ double red[8][256];
     double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     for (int64_t k = threadIdx.x; k < nb; k += blockDim.x)
-        for (int c = 0; c < 7; c++) v[c] += body_part[k * kEnSums + c];
+        for (int c = 0; c < kEnSums; c++) v[c] += body_part[k * kEnSums + c];
     for (int k = threadIdx.x; k < np; k += blockDim.x) v[7] += pair_part[k];
     for (int c = 0; c < 8; c++) red[c][threadIdx.x] = v[c];
     __syncthreads();
@@ -322,14 +305,14 @@ __global__ void k_energy_final(Dev d, int s, int64_t nb, int np, const double* b
     }
 }
 
-void launch_energy(const Dev& d, int sys, const SysInfo& si, int nsm, float4* sa, float4* sb, double* pair_part,
-                   double* body_part, double* out, cudaStream_t s) {
+void launch_energy(const Dev& d, int sys, const SysInfo& si, int nsm, double* pair_part, double* body_part,
+                   double* out, cudaStream_t s) {
     const int64_t nb = si.cap / kEnThreads;
     int grid, run;
     en_shape(si.nb, nsm, grid, run);   // small bodies carry no mass: no pair of theirs adds anything
-    k_energy_body<<<(unsigned)nb, kEnThreads, 0, s>>>(d, si.off, body_part, sa, sb);
-    k_energy_pairs<<<grid, kEnThreads, 0, s>>>(si.nb, si.off, EnSrc{d.x, d.y, d.z, d.m, d.alive, 1}, sa, sb, run,
-                                               body_part, kEnSums, 7, pair_part);
+    k_energy_body<<<(unsigned)nb, kEnThreads, 0, s>>>(d, si.off, body_part);
+    k_energy_pairs<<<grid, kEnThreads, 0, s>>>(si.nb, si.off, EnSrc{d.x, d.y, d.z, d.m, d.alive, 1}, run,
+                                               pair_part);
     k_energy_final<<<1, 256, 0, s>>>(d, sys, nb, grid, body_part, pair_part, out);
 }
 
@@ -346,14 +329,12 @@ void launch_energy(const Dev& d, int sys, const SysInfo& si, int nsm, float4* sa
 constexpr int kNaThreads = 128;
 constexpr int kNaMaxBlocks = 1024;
 constexpr int64_t kNaMaxBodies = (int64_t)kNaThreads * kNaMaxBlocks;   // 131072
-constexpr int kNaSums = 14;   // 1/2 m v^2, m v (3), m/|x|, m x (3), m x x v (3), m, m^2, m |x|
+constexpr int kNaSums = 12;   // 1/2 m v^2, m v (3), m/|x|, m x (3), m x x v (3), m
 constexpr int kNaMaxDevices = 64;
 
 // Every slot a call reads is written earlier in the same call (body block b
-// writes row b and its bodies' float pairs, pair block b writes pair[b]), so
-// nothing here has to start at zero.  4.3 MB of device memory.
+// writes row b, pair block b writes pair[b]), so nothing here has to start at zero.
 struct NaMem {
-    float4 a[kNaMaxBodies], b[kNaMaxBodies];
     double part[kNaMaxBlocks * kNaSums];
     double pair[kEnMaxGrid];
 };
@@ -369,17 +350,12 @@ __global__ void __launch_bounds__(kNaThreads) k_energy_na_body(int64_t n, const 
     if (i < n) {
         const double mi = m[i], xi = x[3 * i], yi = x[3 * i + 1], zi = x[3 * i + 2];
         const double vx = v[3 * i], vy = v[3 * i + 1], vz = v[3 * i + 2];
-        float4 fa, fb;
-        en_split(xi, yi, zi, mi, fa, fb);
-        mem->a[i] = fa;
-        mem->b[i] = fb;
         if (mi != 0.0) {
             s[0] = 0.5 * mi * (vx * vx + vy * vy + vz * vz);
             s[1] = mi * vx;
             s[2] = mi * vy;
             s[3] = mi * vz;
-            const double r = sqrt(xi * xi + yi * yi + zi * zi);
-            s[4] = mi / r;
+            s[4] = mi / sqrt(xi * xi + yi * yi + zi * zi);
             s[5] = mi * xi;
             s[6] = mi * yi;
             s[7] = mi * zi;
@@ -387,8 +363,6 @@ __global__ void __launch_bounds__(kNaThreads) k_energy_na_body(int64_t n, const 
             s[9] = mi * (zi * vx - xi * vz);
             s[10] = mi * (xi * vy - yi * vx);
             s[11] = mi;
-            s[12] = mi * mi;
-            s[13] = mi * r;
         }
     }
     for (int c = 0; c < kNaSums; c++) red[c][threadIdx.x] = s[c];
@@ -404,7 +378,7 @@ __global__ void __launch_bounds__(kNaThreads) k_energy_na_body(int64_t n, const 
 // one block: fixed-order sums of the nb body rows and np pair partials, then E, L, P
 __global__ void __launch_bounds__(256) k_energy_na_final(int nb, int np, double G, double M0, const NaMem* mem,
                                                          double* __restrict__ out) {
-    __shared__ double red[kNaSums + 1][256];   // 30 KB
+    __shared__ double red[kNaSums + 1][256];   // 27 KB
     double s[kNaSums + 1];
     for (int c = 0; c <= kNaSums; c++) s[c] = 0.0;
     for (int b = threadIdx.x; b < nb; b += blockDim.x)
@@ -588,8 +562,7 @@ extern "C" opal_status opal_energy_momentum_noalloc(int64_t n, double G, double 
     if (nb > 0) {
         en_shape(n, nsm, grid, run);
         k_energy_na_body<<<nb, kNaThreads, 0, s>>>(n, m, x, v, mem);
-        k_energy_pairs<<<grid, kNaThreads, 0, s>>>(n, 0, EnSrc{x, x + 1, x + 2, m, nullptr, 3}, mem->a, mem->b, run,
-                                                   mem->part, kNaSums, 11, mem->pair);
+        k_energy_pairs<<<grid, kNaThreads, 0, s>>>(n, 0, EnSrc{x, x + 1, x + 2, m, nullptr, 3}, run, mem->pair);
     }
     k_energy_na_final<<<1, 256, 0, s>>>(nb, grid, G, M0, mem, out);
     cudaError_t rc = cudaGetLastError();

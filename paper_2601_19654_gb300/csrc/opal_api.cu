@@ -98,7 +98,6 @@ struct opal_sim {
     int* d_excnt = nullptr;        // get_state: blocks done with their segments, a system
     int64_t* h_count = nullptr;    // pinned: the live bodies' count, and the arrays of smaller systems (first get_state)
     double* d_en_body = nullptr;
-    float4 *d_en_a = nullptr, *d_en_b = nullptr;   // the energy's float pairs of every body
     double* d_en_pair = nullptr;
     double* d_en_out = nullptr;
     std::vector<void*> allocs;
@@ -615,8 +614,6 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
         CKF(cudaMemsetAsync(s->d_excnt, 0, nsys * sizeof(int), s->stream));
     }
     TRYF(dalloc(s, &s->d_en_body, kEnSums * (N / 128)));
-    TRYF(dalloc(s, &s->d_en_a, N));
-    TRYF(dalloc(s, &s->d_en_b, N));
     TRYF(dalloc(s, &s->d_en_pair, kEnMaxGrid));
     TRYF(dalloc(s, &s->d_en_out, 8));
 
@@ -1061,8 +1058,7 @@ opal_status opal_energy_momentum(const opal_sim* cs, int32_t sys, double* E, dou
     opal_sim* s = const_cast<opal_sim*>(cs);
     if (!s) return set_err(g_err, "sim is NULL"), OPAL_EINVAL;
     if (sys < 0 || sys >= s->d.nsys) return set_err(s->err, "no system %d", sys), OPAL_EINVAL;
-    launch_energy(s->d, sys, s->sys[sys], s->nsm, s->d_en_a, s->d_en_b, s->d_en_pair, s->d_en_body, s->d_en_out,
-                  s->stream);
+    launch_energy(s->d, sys, s->sys[sys], s->nsm, s->d_en_pair, s->d_en_body, s->d_en_out, s->stream);
     CK(cudaGetLastError());
     double o[8];
     CK(cudaMemcpyAsync(o, s->d_en_out, sizeof(o), cudaMemcpyDeviceToHost, s->stream));

@@ -711,12 +711,12 @@ void launch_finish(const Dev& d, cudaStream_t s);
 // Record a one-line reason as the calling thread's last error (opal_last_error(NULL)).
 void set_thread_error(const char* fmt, ...);
 
-// energy, L, P of system sys into out[8]; sa, sb: ntot float4 each, pair_part: kEnMaxGrid
-// doubles, body_part: kEnSums a 128-body block of the largest system
-constexpr int kEnSums = 10;        // sums of a body block
+// energy, L, P of system sys into out[8]; pair_part: kEnMaxGrid doubles, body_part: kEnSums a
+// 128-body block of the largest system
+constexpr int kEnSums = 7;         // sums of a body block
 constexpr int kEnMaxGrid = 1024;   // blocks of the energy's pair sum, one partial each
-void launch_energy(const Dev& d, int sys, const SysInfo& si, int nsm, float4* sa, float4* sb, double* pair_part,
-                   double* body_part, double* out, cudaStream_t s);
+void launch_energy(const Dev& d, int sys, const SysInfo& si, int nsm, double* pair_part, double* body_part, double* out,
+                   cudaStream_t s);
 // get_state of system sys (cap bodies): records (x, y, z, heliocentric v, m, R)
 // and live flags, one a body, into rec and alive; P: 3 doubles of scratch
 // (counter: nsys ints, zero on entry)

@@ -1236,7 +1236,8 @@ void launch_scan(const Dev& d, const PairTile* tiles, int64_t ntiles, int grid, 
     launch_sort_bodies(d, s);
     k_tile_box<<<(unsigned)(d.ntot / kSeg), kSeg, 0, s>>>(d);
     prof_mark("scan: tile boxes");
-    const int64_t cb = (ntiles + 255) / 256;
+    // (no tile pairs where no body has mass: one block, which finds nothing to do)
+    const int64_t cb = ntiles > 0 ? (ntiles + 255) / 256 : 1;
     k_tile_cull<<<(unsigned)(cb < 152 * 8 ? cb : 152 * 8), 256, 0, s>>>(d, tiles, ntiles);
     prof_mark("scan: tile boxes culled");
     k_scan_tiles<<<grid, kSeg, 0, s>>>(d, tiles);
@@ -1250,7 +1251,8 @@ void launch_confirm(const Dev& d, int grid, cudaStream_t s) {
 }
 
 void launch_scan_small(const Dev& d, const PairTile* tiles, int64_t ntiles, bool group, cudaStream_t s) {
-    k_scan_small<<<(unsigned)(ntiles < 1024 ? ntiles : 1024), kSmallThreads, 0, s>>>(d, tiles, (int)ntiles, group ? 1 : 0);
+    const int64_t grid = ntiles < 1 ? 1 : (ntiles < 1024 ? ntiles : 1024);   // (no tile pairs where no body has mass)
+    k_scan_small<<<(unsigned)grid, kSmallThreads, 0, s>>>(d, tiles, (int)ntiles, group ? 1 : 0);
     prof_mark("scan and groups of a small system");
 }
 

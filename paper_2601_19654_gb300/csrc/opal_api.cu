@@ -85,7 +85,8 @@ struct opal_sim {
     PairTile* d_tiles = nullptr;
     int kick_grid = 1, scan_grid = 1, confirm_grid = 1, bs_grid = 1;
     int kick_variant = 0;
-    char kick_desc[256] = {0};
+    char kick_desc[256] = {0};               // the tiled kick in use
+    char kick_desc_small[64] = {0};          // the small systems' (see small_kick)
     int time_kick = 0;                       // graph records events around the kick
     cudaError_t launch_err = cudaSuccess;    // the first failed cluster or cooperative launch of a capture
     int64_t last_involved = 0;               // bodies in encounters in the last step
@@ -727,7 +728,7 @@ opal_status create_impl(const opal_params* p, int32_t nsys, const int64_t* nps, 
                  force ? ", forced" : (best_ms >= 0 ? ", autotuned" : ""));
         CKF(up(d.sys, s->sys.data(), nsys * sizeof(SysInfo)));
         CKF(up(s->d_items, s->items.data(), s->items.size() * sizeof(KickItem)));
-        if (small_kick(s)) snprintf(s->kick_desc, sizeof(s->kick_desc), "mixed, a warp a body, %lld bodies", (long long)ntot);
+        snprintf(s->kick_desc_small, sizeof(s->kick_desc_small), "mixed, a warp a body, %lld bodies", (long long)ntot);
     }
     {
         // warps a position takes in the row sums: eight rows a warp, at most eight warps
@@ -1143,7 +1144,10 @@ opal_status opal_profile_steps(opal_sim* s, int64_t nsteps, int32_t cap, int32_t
 
 const char* opal_last_error(const opal_sim* s) { return s ? s->err : g_err; }
 
-const char* opal_kick_config(const opal_sim* s) { return s ? s->kick_desc : ""; }
+const char* opal_kick_config(const opal_sim* s) {
+    if (!s) return "";
+    return small_kick(s) ? s->kick_desc_small : s->kick_desc;
+}
 
 int32_t opal_graph_kernels(const opal_sim* s) {
     if (!s || !s->graph) return -1;

@@ -90,3 +90,17 @@ def test_small_scan_and_step_against_general(n, n_big, precision):
         tol = np.where(near.any(1), 1e-5 * np.linalg.norm(v, axis=1), tol)
     assert np.all(np.linalg.norm(s["v"] - r["v"], axis=1) <= tol)
     assert np.all(np.linalg.norm(s["x"] - r["x"], axis=1) <= dt * tol + 1e-12)
+
+
+def test_the_kick_named_is_the_one_that_runs(monkeypatch):
+    from paper_2601_19654_gb300 import opal
+    m, x, v, R = _system(500, 500)
+    with opal.Simulation(m, x, v, R, precision=1, dt=0.01) as sim:
+        for order, tiled in (("inorder", False), ("overlap", True), (None, False)):
+            if order:
+                monkeypatch.setenv("OPAL_STEP_ORDER", order)
+            else:
+                monkeypatch.delenv("OPAL_STEP_ORDER")
+            sim.step(1)
+            assert sim.step_overlap == tiled
+            assert sim.kick_config.startswith("mixed t" if tiled else "mixed, a warp a body")

@@ -19,6 +19,8 @@
 // exactly; k_kick_rows adds a body's rows in float-float arithmetic and
 // converts the total to FP64.  FP64 form: the same in doubles, rows summed
 // in FP64.
+#include <cfloat>
+
 #include "opal_internal.cuh"
 
 namespace opal {
@@ -1126,7 +1128,8 @@ __global__ void __launch_bounds__(kSmallKickThreads) k_kick_small(Dev d, int nbl
                 }
             } else {
                 float y = rsqrt_approx(r2);
-                y = fmaf(0.5f * y, fmaf(-(r2 * y), y, 1.0f), y);
+                // (beyond 1.8e19 r2 is infinite and y 0, and stays so; infinity times 0 would be a NaN)
+                y = fmaf(0.5f * y, fmaf(-(fminf(r2, FLT_MAX) * y), y, 1.0f), y);
                 s = (hj[u].w * y) * (y * y);
             }
             tx = fmaf(s, dx, tx);

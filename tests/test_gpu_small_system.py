@@ -104,3 +104,25 @@ def test_the_kick_named_is_the_one_that_runs(monkeypatch):
             sim.step(1)
             assert sim.step_overlap == tiled
             assert sim.kick_config.startswith("mixed t" if tiled else "mixed, a warp a body")
+
+
+# A body so far away that the float square of a separation overflows (beyond 1.8e19), massive or not:
+# it pulls nothing that a float holds, and the others' accelerations are as without it.
+@pytest.mark.parametrize("massive", [True, False])
+@pytest.mark.parametrize("far", [1e18, 1e20, 1e30])
+def test_a_body_beyond_the_float_squares(far, massive):
+    from paper_2601_19654_gb300 import opal
+    m, x, v, R = _system(40, 40)
+    m[-1] = m[-1] if massive else 0.0
+    x[-1], v[-1] = [far, 0.0, 0.0], [0.0, far ** -0.5, 0.0]
+    with opal.Simulation(m, x, v, R, precision=1, dt=0.01) as sim, \
+            opal.Simulation(m[:-1], x[:-1], v[:-1], R[:-1], precision=1, dt=0.01) as ref:
+        a, b = sim.debug_accel(), ref.debug_accel()
+        assert np.array_equal(a[:-1], b)
+        assert np.all(np.abs(a[-1]) <= m.sum() / far ** 2)
+        sim.step(1)
+        ref.step(1)
+        s, r = sim.state(), ref.state()
+    assert s["ids"].tolist() == r["ids"].tolist() + [39]   # (two of the others merge)
+    # (the barycentre's motion takes the far body's momentum: below 1e-5 x its 1e-9 of a velocity)
+    np.testing.assert_allclose(s["x"][:-1], r["x"], rtol=0, atol=1e-12)

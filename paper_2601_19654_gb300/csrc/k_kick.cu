@@ -466,16 +466,21 @@ __global__ void __launch_bounds__(T, MINB) k_kick_mixed(Dev d, const KickItem* _
 // run of the big bodies.
 constexpr double kKickParked = 1.0e150;   // coordinate of lanes without a body (finite squares)
 
+// The high word of a square, for the near test: in the squares' order, but infinity (and a NaN) below all
+// others, so that a pair whose square overflows takes the changeover's path, where 1/r^3 is 0.
+constexpr unsigned kNearZero = 0x80100000u;   // of a zero
+__device__ __forceinline__ unsigned near_word(double r2) { return (unsigned)__double2hiint(r2) + kNearZero; }
+
 struct KickJ {
     double x, y, z, m;
-    int rc2h;   // high word of rc^2 (at least that of 1e-300, so that r = 0 counts as near)
+    unsigned rc2h;   // near_word of rc^2 (at least 1e-300, so that r = 0 counts as near)
 };
 
 __device__ __forceinline__ KickJ kick_load(const Dev& d, int64_t b, bool in) {
-    KickJ r{kKickParked, kKickParked, kKickParked, 0.0, 0};
+    KickJ r{kKickParked, kKickParked, kKickParked, 0.0, kNearZero};
     if (in) {
         const double rc = d.rc[b];
-        r = KickJ{d.x[b], d.y[b], d.z[b], d.m[b], __double2hiint(fmax(rc * rc, 1e-300))};
+        r = KickJ{d.x[b], d.y[b], d.z[b], d.m[b], near_word(fmax(rc * rc, 1e-300))};
     }
     return r;
 }
@@ -488,8 +493,8 @@ __device__ __forceinline__ void kick_pair(const Dev& d, const KickJ& a, double r
     const double dx = j.x - a.x, dy = j.y - a.y, dz = j.z - a.z;
     const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
     double s;
-    if ((unsigned)__double2hiint(r2) <= (unsigned)max(a.rc2h, j.rc2h)) {   // (a NaN is not near)
-        s = slow_pair_d(r2, 1.0, rci, j.rc2h ? d.rc[b] : 0.0, form);
+    if (near_word(r2) <= max(a.rc2h, j.rc2h)) {
+        s = slow_pair_d(r2, 1.0, rci, j.rc2h != kNearZero ? d.rc[b] : 0.0, form);
     } else {
         double y;
         asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));

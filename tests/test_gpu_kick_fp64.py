@@ -84,3 +84,20 @@ def test_fp64_kick_few_items(n, n_big):
         with opal.Simulation(m, x, v, R, precision=0, changeover=form) as sim:
             assert sim.kick_config.startswith("fp64 split")
             _check(sim.debug_accel(rc), m, x, rc, form)
+
+
+# Two massive bodies whose squared separation overflows (and whose own squares do not): the pair
+# adds nothing, as 1/r^3 is 0, and the others' accelerations are as without the two.
+@pytest.mark.parametrize("variant", [0, 1, 2, None])
+def test_fp64_kick_where_a_square_overflows(monkeypatch, variant):
+    from paper_2601_19654_gb300 import opal
+    if variant is not None:
+        monkeypatch.setenv("OPAL_KICK_VARIANT", str(variant))
+    m, x, v, R = _system(140, 140)
+    far = np.arange(140) >= 138
+    x[138], x[139], v[far] = [7e153, 0.0, 0.0], [-7e153, 0.0, 0.0], 0.0
+    with opal.Simulation(m, x, v, R, precision=0) as sim, \
+            opal.Simulation(m[~far], x[~far], v[~far], R[~far], precision=0) as ref:
+        a, b = sim.debug_accel(), ref.debug_accel()
+    assert not a[far].any()
+    np.testing.assert_allclose(a[~far], b, rtol=0, atol=1e-14 * np.abs(b).max())

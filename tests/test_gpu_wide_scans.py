@@ -36,3 +36,28 @@ def test_many_systems_together_as_one_at_a_time(sizes):
     if len(sizes) <= 70:
         assert all(all_stats[key] == total[key] for key in total), (all_stats, total)
     assert len(list(check)) > 0
+
+
+# Slots of a system are padded to 128: 85 systems of 300 bodies have 32640 slots, 86 have 33024 (the group
+# scan's line), 256 of 500 have 32768 buckets, 257 have 32896 (the bucket scan's).  The references are
+# small systems one at a time, which take neither scan.
+@pytest.mark.parametrize("size,count", [(300, 85), (300, 86), (500, 256), (500, 257)])
+def test_counts_at_the_line_as_one_at_a_time(size, count):
+    from paper_2601_19654_gb300 import opal
+    systems = [ic.tiny(2000 + k, size) for k in range(count)]
+    keys = ("n_pairs", "n_groups", "n_candidates", "n_mergers")
+    with opal.Simulation.ensemble(systems, precision=0, dt=0.02) as sim:
+        sim.step(1)
+        together = sim.stats()
+        states = [sim.state(k) for k in range(count)]
+    alone = dict.fromkeys(keys, 0)
+    for s, st in zip(systems, states):
+        with opal.Simulation.from_system(s, precision=0, dt=0.02) as one:
+            one.step(1)
+            stats, ref = one.stats(), one.state()
+        for key in keys:
+            alone[key] += stats[key]
+        assert st["ids"].tolist() == ref["ids"].tolist()
+        np.testing.assert_allclose(st["x"], ref["x"], rtol=0, atol=1e-9)
+    assert alone["n_groups"] > count
+    assert {key: together[key] for key in keys} == alone

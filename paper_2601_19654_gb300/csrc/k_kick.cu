@@ -1200,7 +1200,9 @@ void launch_fp64(const Dev& d, const KickItem* items, int64_t nitems, int grid, 
     k_kick_fp64<W><<<grid, 32 * W, d.kick_smem, s>>>(d, items, nitems);
 }
 // Blocks an SM of the FP64 form: 4 of four warps 4.94 ms on the 16384-body
-// disk, 3: 5.12, 2: 4.99, 5: 4.97 (the pipe is full with two warps a scheduler).
+// disk, 3: 5.12, 2: 4.99, 5: 4.97 (the pipe is full with two warps a scheduler).  Where large super-tiles
+// leave room for fewer (one at 64 tiles of 128 bodies, 196 KB), the grid's other blocks start when
+// the queue is empty and leave at once.
 template <int W>
 int occ_fp64() {
     cudaFuncSetAttribute(k_kick_fp64<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, kKickSuperMax * W * 32 * 24);

@@ -2,23 +2,21 @@
 // (Sec. 3.1, force block, LOOP 2, with the changeover weight K of the hybrid
 // integrator).  G is applied when the partials are reduced.
 //
-// Work is a list of items (i-tile of 128 bodies x a j-range of the same
-// system) that the blocks of a persistent grid take from a queue; each item
-// writes its partial sums to its own row of a buffer that k_kick_rows
-// reduces in a fixed order, so results do not depend on the schedule.
-// j-bodies are staged through shared memory and read by every thread of the
-// block (broadcast).  Pairs closer than 2 (rc_i + rc_max) take a slow path
-// that handles the changeover, the self pair and exact coincidence; all
-// other pairs take the plain Newtonian fast path.
-//
-// Mixed form: FP32 separations of the hi parts of a hi/lo float split of the
-// FP64 positions (the lo parts are added on the slow path), MUFU rsqrt, FP32
-// sums over each 256-body j-tile (the even and the odd j in the two lanes of
-// a packed accumulator), written to the tile's partial row as the float pair
-// (hi, lo) that TwoSum makes of the two lanes, which holds their sum
-// exactly; k_kick_rows adds a body's rows in float-float arithmetic and
-// converts the total to FP64.  FP64 form: the same in doubles, rows summed
-// in FP64.
+// Three forms, each with its own notes below:
+//  - Mixed (k_kick_mixed).  Work is a list of items (a j-tile of 256 bodies against a run of i-tiles of the same
+//    system) that the blocks of a persistent grid take from a queue; each item writes its partial sums to
+//    its own row of a buffer that k_kick_rows reduces in a fixed order, so results do not depend on
+//    the schedule.  j-bodies are staged through shared memory and read by every thread of the block (broadcast).
+//    Pairs closer than 2 (rc_i + rc_max) take a slow path that handles the changeover, the self pair and
+//    exact coincidence; all other pairs take the plain Newtonian fast path: FP32 separations of the hi parts of a
+//    hi/lo float split of the FP64 positions (the lo parts are added on the slow path), MUFU rsqrt, FP32
+//    sums over each 256-body j-tile (the even and the odd j in the two lanes of a packed accumulator), written to
+//    the tile's partial row as the float pair (hi, lo) that TwoSum makes of the two lanes, which holds their sum
+//    exactly; k_kick_rows adds a body's rows in float-float arithmetic and converts the total to FP64.
+//  - FP64 (k_kick_fp64, k_kick_fp64_split).  Items of the same queue, each a pair of tiles of big bodies taken
+//    once for both sides, or small bodies against a run of big ones; the changeover by the pair's own critical
+//    radii; rows of doubles, by body, added in FP64.
+//  - Mixed, one small system (k_kick_small).  A warp a body, no queue and no rows.
 #include <cfloat>
 
 #include "opal_internal.cuh"

@@ -19,8 +19,8 @@ constexpr int kBodyThreads = 128;
 constexpr int kBsMaxMembers = 64;   // bodies per encounter group of the lockstep kernels
 constexpr int64_t kHugeWaitNs = 4000000000;   // the whole-GPU encounter kernel's barrier wait limit (4 s)
 constexpr int kHugeAbortDetail = 2999999;      // status detail of its barrier aborts: this, or this + 1 + group
-constexpr int kKickJTile = 256;
-constexpr int kKickBox = 128;      // positions per tile box of the kick's sorted copies     // j-bodies the kick stages in shared memory at a time
+constexpr int kKickJTile = 256;    // j-bodies the kick stages in shared memory at a time
+constexpr int kKickBox = 128;      // positions per tile box of the kick's sorted copies
 constexpr int kKickSuperMax = 64;  // tiles of a super-tile of the FP64 kick at most
 constexpr int kBsManyGroups = 4864;  // above this many groups a step integrates those of up to 4 members packed, lane per member
 constexpr int kBsSoloGroups = 608;  // above this many groups the small-group kernel makes one attempt at a time
@@ -717,10 +717,9 @@ constexpr int kEnSums = 7;         // sums of a body block
 constexpr int kEnMaxGrid = 1024;   // blocks of the energy's pair sum, one partial each
 void launch_energy(const Dev& d, int sys, const SysInfo& si, int nsm, double* pair_part, double* body_part, double* out,
                    cudaStream_t s);
-// get_state of system sys (cap bodies): records (x, y, z, heliocentric v, m, R)
-// and live flags, one a body, into rec and alive; P: 3 doubles of scratch
-// (counter: nsys ints, zero on entry)
-// get_state: the live bodies' ids, m, R, x and v (9 doubles a slot of the system, see export_view) and their count
+// get_state of system sys (cap slots): the live bodies' ids, m, R, x and v into buf (9 doubles a slot of the
+// system, see export_view) and their count; the second form with scratch (P: 3 doubles, counter: nsys
+// ints, zero between calls, blocks: cap / kBodyThreads ints)
 void launch_export_one(const Dev& d, int sys, int64_t cap, int64_t* count, double* buf, cudaStream_t s);
 void launch_export(const Dev& d, int sys, int64_t cap, double* P, int* counter, int* blocks, int64_t* count, double* buf,
                    cudaStream_t s);

@@ -145,7 +145,7 @@ opal_status opal_get_state(const opal_sim* sim, int32_t sys, int64_t* n_alive, i
 
 /* Total energy E, angular momentum L and momentum P (in democratic
  * heliocentric variables: P = sum m V, barycentric) of system sys, in FP64
- * (the pairs' 1 / r is formed to FP64's precision in other units, its sum in FP64);
+ * (a pair's 1 / r by a computation of the same precision outside the FP64 units);
  * *E_merged_lost is the running sum of the energy removed by mergers, so
  * E + E_merged_lost is the conserved quantity.  Any output may be NULL. */
 opal_status opal_energy_momentum(const opal_sim* sim, int32_t sys, double* E, double L[3],

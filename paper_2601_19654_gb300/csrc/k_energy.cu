@@ -45,9 +45,9 @@ constexpr int kEnShortRun = 32;    // sources of a unit when there are few tiles
 //  - 1 / r = y (1 + d/2 + 3/8 d^2) (the next term is below 2^-61) as the 53-bit mantissa of
 //    a double: y's 24 bits and, 29 places lower, y (d/2 + 3/8 d^2), a product of integers rounded once.
 // Error of 1 / r against 113-bit arithmetic, 200000 pairs for each power of two of r from X down to
-// 2^-12 X: 0.52 to 0.53 x 2^-53 rms and 2.7 x 2^-53 at most, mean below 0.002 x 2^-53 (1 / sqrt of the
-// FP64 square: 0.69 to 0.72, 2.8 and 0.003).
-// A pair closer than 2^-12 X takes the FP64 expression, and so do tiles whose coordinates leave
+// 2^-13 X: 0.52 to 0.53 x 2^-53 rms and 2.7 x 2^-53 at most, mean below 0.002 x 2^-53 (1 / sqrt of the
+// FP64 square: 0.69 to 0.72, 2.8 and 0.004; at 2^-14 X the two rms meet, c's rounding grows as X / r).
+// A pair closer than 2^-13 X takes the FP64 expression, and so do tiles whose coordinates leave
 // the range of the scaling (or are not finite).
 
 // FP64 arrays of the bodies, component c of body i at c[i * stride]; alive may be null
@@ -73,7 +73,7 @@ __device__ __forceinline__ void en_split(double v, double scale, float& a, float
 }
 
 // 1 / |j - i| of two sources j (j2: their nine floats; n: i's, negated), a packed instruction for both where there
-// is one.  Not good (the result means nothing): a separation below 2^-12, zero included, or 1 / r on
+// is one.  Not good (the result means nothing): a separation below 2^-13, zero included, or 1 / r on
 // the other side of a power of two than y, where a mantissa's unit is another (one pair in some 10^6).
 __device__ __forceinline__ void en_recip(const float (&n)[9], const float2 (&j2)[9], double (&out)[2], bool (&good)[2]) {
     auto all = [](float v) { return make_float2(v, v); };
@@ -126,7 +126,7 @@ __device__ __forceinline__ void en_recip(const float (&n)[9], const float2 (&j2)
         const int Y = (int)((yb & 0x7fffffu) | 0x800000u);
         const long long z = ((long long)Y * ch + (long long)(Y >> 2) * cl + (1 << 22)) >> 23;
         const long long y64 = ((long long)yb << 29) + (896LL << 52), u = y64 - z;
-        good[e] = (e ? r2.y : r2.x) >= 0x1p-24f && (u ^ y64) >> 52 == 0;
+        good[e] = (e ? r2.y : r2.x) >= 0x1p-26f && (u ^ y64) >> 52 == 0;
         out[e] = __longlong_as_double(u);
     }
 }
